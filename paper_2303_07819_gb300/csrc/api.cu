@@ -508,15 +508,21 @@ static StepCommon cell_common(ms_model *m, long long i_local, bool scratch_out)
     return sc;
 }
 
-// the cell kernels of a whole coarse interval (FP32 variants 2 and 3): every
-// size class's N0 steps on its own stream, forked once
-static cudaError_t launch_interval_cells(ms_model *m, bool scratch_out)
+// the cell kernels of a run of steps inside one coarse interval (FP32
+// variants 2-5): every size class's steps on its own stream, forked once
+static cudaError_t launch_run_cells(ms_model *m, long long i_local, int nsteps, bool scratch_out)
 {
-    const StepCommon sc = cell_common(m, 0, scratch_out);
+    const StepCommon sc = cell_common(m, i_local, scratch_out);
     cudaError_t e = cell_fork(m->cl, m->stream);
-    if (e == cudaSuccess) e = launch_cell_run32(m->s32, scratch_out ? m->x32 : m->s32, m->P32, sc, m->cl, m->interval);
+    if (e == cudaSuccess) e = launch_cell_run32(m->s32, scratch_out ? m->x32 : m->s32, m->P32, sc, m->cl, nsteps);
     if (e == cudaSuccess) e = cell_join(m->cl, m->stream);
     return e;
+}
+
+// a whole coarse interval of them
+static cudaError_t launch_interval_cells(ms_model *m, bool scratch_out)
+{
+    return launch_run_cells(m, 0, m->interval, scratch_out);
 }
 
 static bool interval_cells(const ms_model *m) { return m->precision == MS_FP32 && m->cl.variant >= 2; }
@@ -1598,12 +1604,18 @@ static int step_enqueue(ms_model *m, double dt, int64_t nsteps)
             Trace ts("msdem.interval start");
             CK(launch_interval_start(m));
         }
+        // What is left of the call or of the interval, whichever ends first.
+        // The FP32 size classes take it as one run: a launch per fine step
+        // would load the floes, build the candidate lists and reduce the
+        // moments at every step.
+        const long long run = interval_cells(m) ? std::min<long long>(nsteps, N - i_local) : 1;
         {
             Trace tf("msdem.fine step");
-            CK(launch_step(m, i_local, false));
+            if (interval_cells(m)) CK(launch_run_cells(m, i_local, (int)run, false));
+            else CK(launch_step(m, i_local, false));
         }
-        m->steps++;
-        nsteps--;
+        m->steps += run;
+        nsteps -= run;
         if (m->steps % N == 0) {
             Trace te("msdem.interval end (coarse step)");
             if (split) {
