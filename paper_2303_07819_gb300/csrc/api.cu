@@ -67,7 +67,7 @@ struct ms_model {
     Phys<float> P32{};
     Phys<double> P64{};
     // layout: stored floe k of cell c at off[c] + ...; orig[k] = caller's index
-    std::vector<int> h_off, h_order, h_cell_of_orig;
+    std::vector<int> h_off, h_order;
     std::vector<long long> h_orig;
     int *d_off = nullptr, *d_order = nullptr;
     // uploads: the caller's arrays as sent ([8][n] FP64), orig and cell of
@@ -227,10 +227,8 @@ static uint32_t to_fix(double frac)
     return (uint32_t)(iv & 0xffffffffLL);
 }
 
-static double from_fix(uint32_t q) { return (double)q * (1.0 / 4294967296.0); }
-
 // f(begin, end) over [0, n) in contiguous chunks on the host's cores (the
-// per-floe loops of uploads, downloads and their checks; each index is
+// per-floe checks of ms_init; each index is
 // handled by exactly one chunk, so the results do not depend on the split)
 template <class F>
 static void host_parallel(long long n, F &&f)
@@ -315,43 +313,17 @@ static UpGeom up_geom(const ms_model *m)
     return g;
 }
 
-// the caller's eight arrays into the pinned stage (all host cores), then to
-// the device's raw copy in one transfer (queued on the model's stream)
-// true if p lies in page-locked host memory of this process (cudaHostAlloc,
-// cudaHostRegister)
-static bool host_pinned(const void *p)
-{
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeHost;
-}
-
-// the caller's eight floe arrays into d_raw on the model's stream: straight
-// from the caller's memory when every array is page-locked, else through the
-// pinned staging buffer array by array (the transfer of one array overlaps
-// the host copy of the next)
+// The caller's eight floe arrays into d_raw on the model's stream, straight
+// from the caller's memory.  Ordinary memory transfers at the rate of
+// page-locked memory where the device reads it through the host's page
+// tables (the Grace host of a GB300: 187 GB/s either way, measured); a copy
+// through a page-locked stage cost the host 60 us per MB first.
 static int send_raw(ms_model *m, const ms_floes *f)
 {
     const long long n = m->n;
     const double *src[8] = {f->x, f->y, f->theta, f->u, f->v, f->omega, f->r, f->h};
-    bool pinned = true;
-    for (int a = 0; a < 8 && pinned; a++) pinned = host_pinned(src[a]);
-    if (pinned) {
-        for (int a = 0; a < 8; a++)
-            CK(cudaMemcpyAsync(m->d_raw + a * n, src[a], sizeof(double) * n, cudaMemcpyHostToDevice, m->stream));
-        return MS_OK;
-    }
-    double *st = (double *)stage(m, sizeof(double) * 8 * n);
-    if (!st) return fail(MS_ERR_CUDA, "cudaMallocHost of %lld bytes failed", (long long)(64 * n));
-    for (int a = 0; a < 8; a++) {
-        host_parallel(n, [&](long long k0, long long k1) {
-            std::memcpy(st + a * n + k0, src[a] + k0, sizeof(double) * (k1 - k0));
-        });
-        CK(cudaMemcpyAsync(m->d_raw + a * n, st + a * n, sizeof(double) * n, cudaMemcpyHostToDevice, m->stream));
-    }
+    for (int a = 0; a < 8; a++)
+        CK(cudaMemcpyAsync(m->d_raw + a * n, src[a], sizeof(double) * n, cudaMemcpyHostToDevice, m->stream));
     return MS_OK;
 }
 
@@ -1479,12 +1451,8 @@ int ms_init(ms_model **out, const ms_grid *grid, const ms_floes *floes, const ms
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(m->h_off.data(), m->d_off, sizeof(int) * (nc + 1), cudaMemcpyDeviceToHost, m->stream);
         std::vector<int> orig32(n);
-        m->h_cell_of_orig.resize(n);
         if (e == cudaSuccess && n > 0)
             e = cudaMemcpyAsync(orig32.data(), m->d_orig, sizeof(int) * n, cudaMemcpyDeviceToHost, m->stream);
-        if (e == cudaSuccess && n > 0)
-            e = cudaMemcpyAsync(m->h_cell_of_orig.data(), m->d_cell_of, sizeof(int) * n, cudaMemcpyDeviceToHost,
-                                m->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
         release();
         if (e != cudaSuccess) {
@@ -1633,11 +1601,8 @@ static int step_enqueue(ms_model *m, double dt, int64_t nsteps)
 int ms_moments(ms_model *m, double *out)
 {
     if (!m || !out) return fail(MS_ERR_ARG, "NULL argument");
-    double *st = (double *)stage(m, sizeof(double) * m->ncell * NMOM);
-    if (!st) return fail(MS_ERR_CUDA, "cudaMallocHost failed");
-    CK(cudaMemcpyAsync(st, m->d_mom, sizeof(double) * m->ncell * NMOM, cudaMemcpyDeviceToHost, m->stream));
+    CK(cudaMemcpyAsync(out, m->d_mom, sizeof(double) * m->ncell * NMOM, cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
-    std::memcpy(out, st, sizeof(double) * m->ncell * NMOM);
     return MS_OK;
 }
 
@@ -1662,54 +1627,15 @@ int ms_coupling(ms_model *m, double *q, double *targets, double *window, int64_t
 static int download(ms_model *m, bool truth, double *out)
 {
     Trace tr("msdem.get_floes");
-    const long long n = m->n;
-    if (n == 0) return MS_OK;
-    const int nx = m->g.nx;
-    if (m->precision == MS_FP64) {
-        double *st = (double *)stage(m, sizeof(double) * 8 * n);
-        if (!st) return fail(MS_ERR_CUDA, "cudaMallocHost failed");
-        const DevState64 &s = truth ? m->t64[m->tcur] : m->s64;
-        const double *src[8] = {s.x, s.y, s.th, s.u, s.v, s.w, s.r, s.h};
-        for (int a = 0; a < 8; a++)
-            CK(cudaMemcpyAsync(st + a * n, src[a], sizeof(double) * n, cudaMemcpyDeviceToHost, m->stream));
-        CK(cudaStreamSynchronize(m->stream));
-        host_parallel(n, [&](long long k0, long long k1) {
-            for (long long k = k0; k < k1; k++) {
-                const long long l = truth ? k : m->h_orig[k];
-                const int c = truth ? 0 : m->h_cell_of_orig[l];
-                const double X0 = truth ? 0.0 : (c % nx) * m->g.Lcx, Y0 = truth ? 0.0 : (c / nx) * m->g.Lcy;
-                out[l] = X0 + st[k];
-                out[n + l] = Y0 + st[n + k];
-                for (int a = 2; a < 8; a++) out[a * n + l] = st[a * n + k];
-            }
-        });
-    } else {
-        unsigned char *st = (unsigned char *)stage(m, sizeof(float) * 8 * n);
-        if (!st) return fail(MS_ERR_CUDA, "cudaMallocHost failed");
-        uint32_t *qx = (uint32_t *)st, *qy = qx + n;
-        float *fl = (float *)(qy + n);
-        const DevState32 &s = truth ? m->t32[m->tcur] : m->s32;
-        CK(cudaMemcpyAsync(qx, s.xq, 4 * n, cudaMemcpyDeviceToHost, m->stream));
-        CK(cudaMemcpyAsync(qy, s.yq, 4 * n, cudaMemcpyDeviceToHost, m->stream));
-        const float *src[6] = {s.th, s.u, s.v, s.w, s.r, s.h};
-        for (int a = 0; a < 6; a++)
-            CK(cudaMemcpyAsync(fl + a * n, src[a], 4 * n, cudaMemcpyDeviceToHost, m->stream));
-        CK(cudaStreamSynchronize(m->stream));
-        host_parallel(n, [&](long long k0, long long k1) {
-            for (long long k = k0; k < k1; k++) {
-                const long long l = truth ? k : m->h_orig[k];
-                if (truth) {
-                    out[l] = from_fix(qx[k]) * m->g.Lx;
-                    out[n + l] = from_fix(qy[k]) * m->g.Ly;
-                } else {
-                    const int c = m->h_cell_of_orig[l];
-                    out[l] = ((c % nx) + from_fix(qx[k])) * m->g.Lcx;
-                    out[n + l] = ((c / nx) + from_fix(qy[k])) * m->g.Lcy;
-                }
-                for (int a = 0; a < 6; a++) out[(a + 2) * n + l] = fl[a * n + k];
-            }
-        });
-    }
+    if (m->n == 0) return MS_OK;
+    const UpGeom g = up_geom(m);
+    const int *orig = truth ? nullptr : m->d_orig;
+    if (m->precision == MS_FP64)
+        CK(launch_cells_to_floes64(truth ? m->t64[m->tcur] : m->s64, orig, m->d_cell_of, g, m->d_raw, m->stream));
+    else
+        CK(launch_cells_to_floes32(truth ? m->t32[m->tcur] : m->s32, orig, m->d_cell_of, g, m->d_raw, m->stream));
+    CK(cudaMemcpyAsync(out, m->d_raw, sizeof(double) * 8 * m->n, cudaMemcpyDeviceToHost, m->stream));
+    CK(cudaStreamSynchronize(m->stream));
     return MS_OK;
 }
 
@@ -1731,6 +1657,8 @@ int ms_truth_get_floes(ms_model *m, double *out)
     return download(m, true, out);
 }
 
+// The floes in the caller's order, converted on the device (into the buffer
+// that uploads arrive in) and copied straight into the caller's memory.
 int ms_set_floes(ms_model *m, const ms_floes *floes)
 {
     if (!m) return fail(MS_ERR_ARG, "model is NULL");
@@ -1808,11 +1736,8 @@ int ms_truth_moments(ms_model *m, double *out)
     a.fd = m->d_fd;
     if (m->precision == MS_FP64) CK(launch_truth_moments64(m->t64[m->tcur], m->P64, a, m->cb, m->d_tmom, m->stream));
     else CK(launch_truth_moments32(m->t32[m->tcur], m->P32, a, m->cb, m->d_tmom, m->stream));
-    double *st = (double *)stage(m, sizeof(double) * m->ncell * NMOM);
-    if (!st) return fail(MS_ERR_CUDA, "cudaMallocHost failed");
-    CK(cudaMemcpyAsync(st, m->d_tmom, sizeof(double) * m->ncell * NMOM, cudaMemcpyDeviceToHost, m->stream));
+    CK(cudaMemcpyAsync(out, m->d_tmom, sizeof(double) * m->ncell * NMOM, cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
-    std::memcpy(out, st, sizeof(double) * m->ncell * NMOM);
     return MS_OK;
 }
 

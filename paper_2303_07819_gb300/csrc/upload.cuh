@@ -40,4 +40,12 @@ cudaError_t launch_floes_to_cells32(const double *raw, const int *orig, const in
 cudaError_t launch_floes_to_cells64(const double *raw, const int *orig, const int *cell_of, UpGeom g,
                                     DevState64 s, cudaStream_t st);
 
+// out = device [8][n] doubles as raw: stored floe k goes to caller's floe
+// orig[k] of cell cell_of[orig[k]]; orig NULL (the truth DEM): floe k is the
+// caller's k, its position in domain coordinates
+cudaError_t launch_cells_to_floes32(const DevState32 &s, const int *orig, const int *cell_of, UpGeom g, double *out,
+                                    cudaStream_t st);
+cudaError_t launch_cells_to_floes64(const DevState64 &s, const int *orig, const int *cell_of, UpGeom g, double *out,
+                                    cudaStream_t st);
+
 }  // namespace msd

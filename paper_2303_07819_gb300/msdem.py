@@ -235,12 +235,12 @@ class Model:
         _check(load().ms_sync(self._h))
 
     def moments(self) -> np.ndarray:
-        out = np.zeros((self.ncell, NMOM))
+        out = np.empty((self.ncell, NMOM))
         _check(load().ms_moments(self._h, _ptr(out)))
         return out
 
     def floes(self) -> dict:
-        out = np.zeros((8, self.n))
+        out = np.empty((8, self.n))
         _check(load().ms_get_floes(self._h, _ptr(out)))
         return {k: out[i] for i, k in enumerate(FLOE_KEYS)}
 
@@ -250,7 +250,7 @@ class Model:
 
     def coupling(self) -> dict:
         nc = self.ncell
-        q = np.zeros((4, nc)); tg = np.zeros((4, nc)); win = np.zeros((NWIN, nc))
+        q, tg, win = np.empty((4, nc)), np.empty((4, nc)), np.empty((NWIN, nc))
         fl = np.zeros(3, dtype=np.int64)
         _check(load().ms_coupling(self._h, _ptr(q), _ptr(tg), _ptr(win),
                                   fl.ctypes.data_as(C.POINTER(C.c_int64))))
@@ -261,12 +261,12 @@ class Model:
         _check(load().ms_truth_step(self._h, float(dt), int(nsteps)))
 
     def truth_moments(self) -> np.ndarray:
-        out = np.zeros((self.ncell, NMOM))
+        out = np.empty((self.ncell, NMOM))
         _check(load().ms_truth_moments(self._h, _ptr(out)))
         return out
 
     def truth_floes(self) -> dict:
-        out = np.zeros((8, self.n))
+        out = np.empty((8, self.n))
         _check(load().ms_truth_get_floes(self._h, _ptr(out)))
         return {k: out[i] for i, k in enumerate(FLOE_KEYS)}
 
