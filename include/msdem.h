@@ -262,7 +262,7 @@ int ms_set_resident(ms_model *m, double skin_steps, int32_t block_floes);
  * 4 kernel variant, 5 threads per block, 6 bin width (per mille of the mean
  * floe spacing), 7 cell-kernel launches per coarse interval (msDEM, whole
  * intervals, no coarse step),
- * 8 kernels per coarse step, 9 kernels per truth step, 10 steps done,
+ * 8 kernels per coarse step, 9 kernels per call of truth steps (each up to 256 steps), 10 steps done,
  * 11 truth steps done, 12 graph replays so far, 13 contacts seen deeper than
  * half the smaller radius, 14 persistent launch, 15 LF substeps of the last
  * coarse step, 16 skin horizon of variant 5 in thousandths of a fine step,

@@ -92,6 +92,7 @@ struct ms_model {
     int tcur = 0;
     void *d_fd = nullptr;
     TruthBins tb{}, cb{};
+    unsigned char *d_twork = nullptr;   // the truth steps' work arrays (made by the first of them)
     double *d_tmom = nullptr;
     // schedule
     long long steps = 0, truth_steps = 0;
@@ -1035,6 +1036,7 @@ static int setup_truth_bins(ms_model *m, const double *r, double rmax)
         b.nbx2 = dims[k][2];
         b.nby2 = dims[k][3];
         b.r_split = k == 0 ? (float)(best_q * rmax) : 0.0f;
+        b.r_max = (float)rmax;
         const int nbins = b.nbins();
         b.nscan_blocks = (nbins + 1023) / 1024;
         if (b.nscan_blocks > 1024) return fail(MS_ERR_ARG, "too many bins (%d)", nbins);
@@ -1624,6 +1626,8 @@ int ms_coupling(ms_model *m, double *q, double *targets, double *window, int64_t
     return MS_OK;
 }
 
+// The floes in the caller's order, converted on the device (into the buffer
+// that uploads arrive in) and copied straight into the caller's memory.
 static int download(ms_model *m, bool truth, double *out)
 {
     Trace tr("msdem.get_floes");
@@ -1657,8 +1661,6 @@ int ms_truth_get_floes(ms_model *m, double *out)
     return download(m, true, out);
 }
 
-// The floes in the caller's order, converted on the device (into the buffer
-// that uploads arrive in) and copied straight into the caller's memory.
 int ms_set_floes(ms_model *m, const ms_floes *floes)
 {
     if (!m) return fail(MS_ERR_ARG, "model is NULL");
@@ -1691,18 +1693,33 @@ int ms_set_floes(ms_model *m, const ms_floes *floes)
     return MS_OK;
 }
 
-static cudaError_t truth_one(ms_model *m, int cur, int nxt, long long step)
+static TruthArgs truth_args(const ms_model *m, double dt, long long step)
 {
     TruthArgs a;
     a.n = m->n;
     a.g = m->g;
-    a.k = geo32(m->g.Lx, m->g.Ly, 1, 1, m->truth_dt);
-    a.dt = m->truth_dt;
+    a.k = geo32(m->g.Lx, m->g.Ly, 1, 1, dt);
+    a.iLx = 1.0 / m->g.Lx;
+    a.iLy = 1.0 / m->g.Ly;
+    a.dt = dt;
     a.step = step;
     a.ctrl = m->d_ctrl;
     a.fd = m->d_fd;
-    if (m->precision == MS_FP64) return launch_truth_step64(m->t64[cur], m->t64[nxt], m->P64, a, m->tb, m->stream);
-    return launch_truth_step32(m->t32[cur], m->t32[nxt], m->P32, a, m->tb, m->stream);
+    return a;
+}
+
+// nsteps <= TRUTH_CHUNK truth steps from copy cur to the other, step `step` first
+static cudaError_t truth_run(ms_model *m, int cur, long long step, int nsteps)
+{
+    if (!m->d_twork) {
+        cudaError_t e = dalloc(m, &m->d_twork, truth_work_bytes(m->precision, m->n, m->P64, m->g));
+        if (e == cudaSuccess) e = truth_work_init(m->precision, m->n, m->P64, m->g, m->d_twork, m->stream);
+        if (e != cudaSuccess) return e;
+    }
+    const TruthArgs a = truth_args(m, m->truth_dt, step);
+    if (m->precision == MS_FP64)
+        return launch_truth_run64(m->t64[cur], m->t64[1 - cur], m->P64, a, m->tb, m->d_twork, nsteps, m->stream);
+    return launch_truth_run32(m->t32[cur], m->t32[1 - cur], m->P32, m->P64, a, m->tb, m->d_twork, nsteps, m->stream);
 }
 
 int ms_truth_step(ms_model *m, double dt, int64_t nsteps)
@@ -1714,10 +1731,12 @@ int ms_truth_step(ms_model *m, double dt, int64_t nsteps)
     if (m->truth_dt == 0.0) m->truth_dt = dt;
     else if (dt != m->truth_dt) return fail(MS_ERR_ARG, "dt differs from the truth model's dt");
     Trace tr("msdem.truth steps");
-    for (long long k = 0; k < nsteps; k++) {
-        CK(truth_one(m, m->tcur, 1 - m->tcur, m->truth_steps));
+    while (nsteps > 0) {
+        const int k = (int)std::min<int64_t>(nsteps, TRUTH_CHUNK);
+        CK(truth_run(m, m->tcur, m->truth_steps, k));
         m->tcur = 1 - m->tcur;
-        m->truth_steps++;
+        m->truth_steps += k;
+        nsteps -= k;
     }
     return read_errors(m);
 }
@@ -1726,14 +1745,7 @@ int ms_truth_moments(ms_model *m, double *out)
 {
     if (!m || !out) return fail(MS_ERR_ARG, "NULL argument");
     if (no_truth(m)) return MS_ERR_STATE;
-    TruthArgs a;
-    a.n = m->n;
-    a.g = m->g;
-    a.k = geo32(m->g.Lx, m->g.Ly, 1, 1, m->truth_dt > 0 ? m->truth_dt : 1.0);
-    a.dt = m->truth_dt;
-    a.step = m->truth_steps;
-    a.ctrl = m->d_ctrl;
-    a.fd = m->d_fd;
+    const TruthArgs a = truth_args(m, m->truth_dt > 0 ? m->truth_dt : 1.0, m->truth_steps);
     if (m->precision == MS_FP64) CK(launch_truth_moments64(m->t64[m->tcur], m->P64, a, m->cb, m->d_tmom, m->stream));
     else CK(launch_truth_moments32(m->t32[m->tcur], m->P32, a, m->cb, m->d_tmom, m->stream));
     CK(cudaMemcpyAsync(out, m->d_tmom, sizeof(double) * m->ncell * NMOM, cudaMemcpyDeviceToHost, m->stream));
@@ -1785,7 +1797,7 @@ int ms_time_kernel(ms_model *m, int32_t which, double dt, int32_t reps, double *
         else if (which == 2 && interval_cells(m)) le = launch_interval_cells(m, true);
         else if (which == 2)
             for (int i = 0; i < m->interval && le == cudaSuccess; i++) le = launch_step(m, i, true);
-        else le = truth_one(m, m->tcur, 1 - m->tcur, m->truth_steps);
+        else le = truth_run(m, m->tcur, m->truth_steps, 1);
     }
     if (le == cudaSuccess) le = cudaEventRecord(e1, m->stream);
     if (le == cudaSuccess) le = cudaEventSynchronize(e1);
@@ -1901,7 +1913,7 @@ int ms_info(ms_model *m, int64_t *out)
     out[6] = (int64_t)std::lround(m->cl.bin_beta * 1000.0f);
     out[7] = interval_launches(m);
     out[8] = m->fc.couple ? coarse_launches() : 1;
-    out[9] = truth_launches(m->tb);
+    out[9] = 1;
     out[10] = m->steps;
     out[11] = m->truth_steps;
     out[12] = m->replays;

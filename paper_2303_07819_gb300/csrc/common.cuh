@@ -436,7 +436,7 @@ int coarse_launches();
 struct TruthBins {
     int nbx, nby;          // bins per side (1 x 1: brute force)
     int nbx2, nby2;        // the large floes' grid
-    float r_split;
+    float r_split, r_max;
     __host__ __device__ int nbins() const { return nbx * nby + nbx2 * nby2; }
     int *count;            // [nbins]
     int *start;            // [nbins + 1]
@@ -450,20 +450,27 @@ struct TruthArgs {
     long long n;
     Geom g;
     Geo32 k;               // domain-sized constants (fixed point of the domain)
+    double iLx, iLy;       // 1 / g.Lx, 1 / g.Ly
     double dt;
     long long step;        // steps done before this one
     Ctrl *ctrl;            // error bits and deep-overlap counter
     void *fd;              // [3][n] drag of the last step (R)
 };
-cudaError_t launch_truth_step32(const DevState32 &in, const DevState32 &out, const Phys<float> &P,
-                                const TruthArgs &a, TruthBins &b, cudaStream_t st);
-cudaError_t launch_truth_step64(const DevState64 &in, const DevState64 &out, const Phys<double> &P,
-                                const TruthArgs &a, TruthBins &b, cudaStream_t st);
+// truth_run.cu: nsteps <= TRUTH_CHUNK steps from `in` to `out` in one launch.
+// work: truth_work_bytes of device memory, made ready once by
+// truth_work_init; between launches it holds only what that made (the FP64
+// ocean's table, which depends on the forcing alone).
+constexpr int TRUTH_CHUNK = 256;
+size_t truth_work_bytes(int precision, long long n, const Phys<double> &P, const Geom &g);
+cudaError_t truth_work_init(int precision, long long n, const Phys<double> &P, const Geom &g, void *work, cudaStream_t st);
+cudaError_t launch_truth_run32(const DevState32 &in, const DevState32 &out, const Phys<float> &P, const Phys<double> &P64,
+                               const TruthArgs &a, TruthBins &b, void *work, int nsteps, cudaStream_t st);
+cudaError_t launch_truth_run64(const DevState64 &in, const DevState64 &out, const Phys<double> &P, const TruthArgs &a,
+                               TruthBins &b, void *work, int nsteps, cudaStream_t st);
 cudaError_t launch_truth_moments32(const DevState32 &s, const Phys<float> &P, const TruthArgs &a,
                                    TruthBins &cells, double *mom, cudaStream_t st);
 cudaError_t launch_truth_moments64(const DevState64 &s, const Phys<double> &P, const TruthArgs &a,
                                    TruthBins &cells, double *mom, cudaStream_t st);
-int truth_launches(const TruthBins &b);
 // per-cell moments with scratch from a static device array (no allocation)
 long long noalloc_max_floes();
 int noalloc_max_cells();

@@ -1,0 +1,636 @@
+// truth_run.cu -- up to TRUTH_CHUNK steps of the un-localised DEM (Sec. 4) in
+// one cooperative launch, FP32 and FP64.
+//
+// What bounded it: nine launches a step (clear, bin, three-pass scan, scatter,
+// sort, contacts) to find again contacts that last many steps, and in the
+// contact kernel the latency of bin -> index -> partner loads.  A floe moves a
+// metre a step against radii of hundreds, so it keeps a candidate list, its
+// partners within r_l + s_l + r_j + s_j (s: the floe's skin), until some floe
+// has moved farther than its skin; a step is then one pass over the lists and
+// one grid barrier.  A rebuild costs four barriers: count, block sums, starts,
+// scatter (positions and reaches copied in bin order, so a search reads
+// consecutive memory), search.
+//
+// Lists are in ascending floe order and hold every floe that can touch, so a
+// floe's force is the sum over its contacts in ascending partner order
+// whenever the lists were built: splitting a run of steps differently, or
+// resuming it, changes no bit.  Floes of radius <= r_split and larger ones sit
+// in separate grids of bins, as the host chose them (setup_truth_bins).
+//
+// Measured (65,341 power-law floes, FP32): 87 us a step as nine launches.
+#include <climits>
+#include <cooperative_groups.h>
+
+#include "common.cuh"
+#include "truth_step.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace msd {
+
+namespace {
+
+constexpr int TT = 256;       // threads per block
+constexpr int LT = 64;        // candidates per floe; a floe with more searches its bins at every step
+
+// a floe in the working copy: what a contact test reads, and the rest
+struct A32 { uint32_t x, y; float r, h; };
+struct A64 { double x, y, r, h; };
+template <class R> struct Rest { R u, v, w, th; };
+
+struct Tr32 {
+    using R = float;
+    using A = A32;
+    using State = DevState32;
+};
+struct Tr64 {
+    using R = double;
+    using A = A64;
+    using State = DevState64;
+};
+
+struct Sorted { uint32_t x, y; float reach; int l; };   // a floe in bin order
+
+template <class T>
+struct Work {
+    typename T::A *A[2];
+    Rest<typename T::R> *B[2];
+    int *binof, *rank, *cnt, *list;    // [n], [n], [n], [LT][n]
+    uint2 *xb;                         // [n] position at the build, fixed point of the domain
+    float *skin;                       // [n]
+    Sorted *sorted;                    // [n]
+    int *bsum;                         // [gridDim]
+    int *ctl;                          // flags [3], largest skin [2], sum of speeds [2] (float bits)
+    double2 *wind;                     // [TRUTH_CHUNK]
+    double2 *tile;                     // FP64: [ty][tx][n_modes] cos, sin of each mode at the tiles' centres
+    int tx, ty;                        // 0: no table
+};
+
+__device__ __forceinline__ A32 load_a(const DevState32 &s, long long l) { return {s.xq[l], s.yq[l], s.r[l], s.h[l]}; }
+__device__ __forceinline__ A64 load_a(const DevState64 &s, long long l) { return {s.x[l], s.y[l], s.r[l], s.h[l]}; }
+__device__ __forceinline__ void store_xy(const DevState32 &s, long long l, const A32 &a) { s.xq[l] = a.x; s.yq[l] = a.y; }
+__device__ __forceinline__ void store_xy(const DevState64 &s, long long l, const A64 &a) { s.x[l] = a.x; s.y[l] = a.y; }
+
+// 32-bit fixed point of the domain
+__device__ __forceinline__ uint2 fixed(const A32 &a, const Geom &) { return make_uint2(a.x, a.y); }
+__device__ __forceinline__ uint32_t fixed1(double x, double L)
+{
+    const double q = floor(x / L * 4294967296.0);
+    return (uint32_t)(long long)fmin(fmax(q, 0.0), 4294967295.0);   // a wall's own coordinate is L
+}
+__device__ __forceinline__ uint2 fixed(const A64 &a, const Geom &g)
+{
+    return make_uint2(fixed1(a.x, g.Lx), fixed1(a.y, g.Ly));
+}
+
+// fixed-point separation in metres: the periodic minimum image, or between
+// walls the plain difference
+__device__ __forceinline__ float sep_x(uint32_t a, uint32_t b, float sx, bool walls)
+{
+    return walls ? (float)((long long)a - (long long)b) * sx : (float)(int)(a - b) * sx;
+}
+
+__device__ __forceinline__ int fbin(uint32_t q, int nb) { return (int)(((unsigned long long)q * (unsigned)nb) >> 32); }
+
+// Calls f(first, last + 1) for the ranges of sorted floes in the bins of one
+// grid (nbx x nby bins from bin `base`) within (rx, ry) bin sides of the bin
+// that holds a floe at fixed point q; bins side by side in x are one range.
+template <class F>
+__device__ __forceinline__ void visit_ranges(const int *start, int base, int nbx, int nby, uint2 q, float rx, float ry,
+                                             bool walls, F &&f)
+{
+    // margin against rounding; NaN (a diverged state) takes every bin
+    const int kx = rx * 1.0001f < (float)nbx ? (int)ceilf(rx * 1.0001f) : nbx;
+    const int ky = ry * 1.0001f < (float)nby ? (int)ceilf(ry * 1.0001f) : nby;
+    const int bx = fbin(q.x, nbx), by = fbin(q.y, nby);
+    const bool allx = 2 * kx + 1 >= nbx, ally = 2 * ky + 1 >= nby;
+    const int rows = ally ? nby : 2 * ky + 1;
+    for (int i = 0; i < rows; i++) {
+        int cy = ally ? i : by - ky + i;
+        cy = cy < 0 ? cy + nby : (cy >= nby ? cy - nby : cy);
+        const int *row = start + base + cy * nbx;
+        if (allx) {
+            f(row[0], row[nbx]);
+            continue;
+        }
+        const int lo = bx - kx, hi = bx + kx;
+        f(row[max(lo, 0)], row[min(hi, nbx - 1) + 1]);
+        if (!walls) {
+            if (lo < 0) f(row[lo + nbx], row[nbx]);
+            if (hi >= nbx) f(row[0], row[hi - nbx + 1]);
+        }
+    }
+}
+
+// ascending sort of v[0..N) in registers (bitonic, every index static)
+template <int N>
+__device__ __forceinline__ void sort_net(int (&v)[N])
+{
+#pragma unroll
+    for (int k = 2; k <= N; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int i = 0; i < N; i++) {
+                const int o = i ^ j;
+                if (o > i) {
+                    const int a = v[i], b = v[o];
+                    const bool up = (i & k) == 0;
+                    v[i] = up ? min(a, b) : max(a, b);
+                    v[o] = up ? max(a, b) : min(a, b);
+                }
+            }
+}
+
+// (not inlined: the registers are the sort's own)
+template <int N>
+__device__ __noinline__ void sort_list(int *list, long long n, int cnt)
+{
+    int v[N];
+#pragma unroll
+    for (int i = 0; i < N; i++) v[i] = i < cnt ? list[i * n] : INT_MAX;
+    sort_net(v);
+#pragma unroll
+    for (int i = 0; i < N; i++)
+        if (i < cnt) list[i * n] = v[i];
+}
+
+// separation of partner a from floe o in the state's own precision
+__device__ __forceinline__ void pair_xy(const A32 &a, const A32 &o, const TruthArgs &t, bool walls, float &dx, float &dy)
+{
+    dx = sep_x(a.x, o.x, t.k.sx, walls);
+    dy = (float)(int)(a.y - o.y) * t.k.sy;
+}
+__device__ __forceinline__ void pair_xy(const A64 &a, const A64 &o, const TruthArgs &t, bool walls, double &dx, double &dy)
+{
+    dx = a.x - o.x;
+    dy = a.y - o.y;
+    if (!walls) dx -= t.g.Lx * rint(dx * t.iLx);
+    dy -= t.g.Ly * rint(dy * t.iLy);
+}
+
+// the current at a floe: FP32 from the phases in cycles per domain
+__device__ __forceinline__ void ocean_at(const Phys<float> &P, const Work<Tr32> &, const TruthArgs &, const A32 &a,
+                                         float &uo, float &vo, float &zeta)
+{
+    const float xf = (float)a.x * INV2_32F, yf = (float)a.y * INV2_32F;
+    uo = P.uo_x; vo = P.uo_y; zeta = 0.0f;
+    for (int m = 0; m < P.n_modes; m++) {
+        float cyc = P.kdx[m] * xf + P.kdy[m] * yf + P.mCyc[m];
+        cyc -= floorf(cyc);
+        float s, c;
+        sincospif(2.0f * cyc, &s, &c);
+        uo -= P.mAu[m] * c;
+        vo += P.mAv[m] * c;
+        zeta -= P.mAz[m] * s;
+    }
+}
+
+// FP64: each mode's sine and cosine at the centre of the floe's tile turned by
+// the angle to the floe, at most a quarter radian, by Taylor sums (remainder
+// below 2^-56): 13 FP64 operations where a sincos takes about 60.  Which
+// tile, and so the rounding, is a matter of the position alone.
+__device__ __forceinline__ void ocean_at(const Phys<double> &P, const Work<Tr64> &w, const TruthArgs &t, const A64 &a,
+                                         double &uo, double &vo, double &zeta)
+{
+    if (w.tx == 0) {
+        ocean_f64(P, a.x, a.y, uo, vo, zeta);
+        return;
+    }
+    const int ix = min((int)(a.x * t.iLx * w.tx), w.tx - 1), iy = min((int)(a.y * t.iLy * w.ty), w.ty - 1);
+    const double dx = a.x - (ix + 0.5) * (t.g.Lx / w.tx), dy = a.y - (iy + 0.5) * (t.g.Ly / w.ty);
+    const double2 *ref = w.tile + ((size_t)max(iy, 0) * w.tx + max(ix, 0)) * P.n_modes;
+    uo = P.uo_x; vo = P.uo_y; zeta = 0.0;
+    for (int m = 0; m < P.n_modes; m++) {
+        const double th = P.mKx[m] * dx + P.mKy[m] * dy, t2 = th * th;
+        const double2 r = ref[m];
+        double ps = fma(t2, fma(t2, fma(t2, fma(t2, -1.0 / 39916800.0, 1.0 / 362880.0), -1.0 / 5040.0), 1.0 / 120.0),
+                        -1.0 / 6.0);
+        ps = fma(ps * t2, th, th);
+        double pc = fma(t2, fma(t2, fma(t2, fma(t2, fma(t2, 1.0 / 479001600.0, -1.0 / 3628800.0), 1.0 / 40320.0),
+                                        -1.0 / 720.0), 1.0 / 24.0), -0.5);
+        pc = fma(pc, t2, 1.0);
+        const double c = r.x * pc - r.y * ps, s = r.y * pc + r.x * ps;
+        uo -= P.mAu[m] * c;
+        vo += P.mAv[m] * c;
+        zeta -= P.mAz[m] * s;
+    }
+}
+
+__global__ void k_truth_tiles(Phys<double> P, Geom g, Work<Tr64> w)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= w.tx * w.ty * P.n_modes) return;
+    const int m = i % P.n_modes, tile = i / P.n_modes;
+    const double x = (tile % w.tx + 0.5) * (g.Lx / w.tx), y = (tile / w.tx + 0.5) * (g.Ly / w.ty);
+    double s, c;
+    sincos(P.mKx[m] * x + P.mKy[m] * y + P.mPh[m], &s, &c);
+    w.tile[i] = make_double2(c, s);
+}
+
+// tiles small enough that no mode turns by more than 1/8 from a tile's centre
+// along either axis (none if that takes more than 64 MB)
+void tile_counts(const Phys<double> &P, const Geom &g, int &tx, int &ty)
+{
+    double ax = 0.0, ay = 0.0;
+    for (int m = 0; m < P.n_modes; m++) {
+        ax = fmax(ax, fabs(P.mKx[m]) * g.Lx);
+        ay = fmax(ay, fabs(P.mKy[m]) * g.Ly);
+    }
+    const double nx = ceil(4.0 * ax) + 1.0, ny = ceil(4.0 * ay) + 1.0;
+    const bool fits = P.n_modes > 0 && nx * ny * P.n_modes <= 4194304.0;
+    tx = fits ? (int)nx : 0;
+    ty = fits ? (int)ny : 0;
+}
+
+__device__ __forceinline__ void wall_force(const A32 &a, const TruthArgs &t, float u, float v, float w, const Phys<float> &P,
+                                           float &fx, float &fy, float &tq, unsigned &deep)
+{
+    // distances to the walls from the fixed point: exact integers, one rounding
+    wall_add((float)a.x * t.k.sx, (float)(4294967296ll - (long long)a.x) * t.k.sx, u, v, w, a.r, a.h, P, fx, fy, tq, deep);
+}
+__device__ __forceinline__ void wall_force(const A64 &a, const TruthArgs &t, double u, double v, double w,
+                                           const Phys<double> &P, double &fx, double &fy, double &tq, unsigned &deep)
+{
+    wall_add(a.x, t.g.Lx - a.x, u, v, w, a.r, a.h, P, fx, fy, tq, deep);
+}
+
+// forward Euler on the position; reading: a centre that would pass a wall
+// stays on it (in a stable run the wall's contact force stops the floe long
+// before)
+__device__ __forceinline__ A32 moved(const A32 &a, const TruthArgs &t, bool walls, float u, float v)
+{
+    A32 b = a;
+    const float dt = t.k.dt;
+    if (walls) {
+        long long xn = (long long)a.x + __float2int_rn(dt * u * t.k.isx);
+        xn = xn < 0 ? 0 : (xn > 4294967295ll ? 4294967295ll : xn);
+        b.x = (uint32_t)xn;
+    } else {
+        b.x = a.x + (uint32_t)__float2int_rn(dt * u * t.k.isx);
+    }
+    b.y = a.y + (uint32_t)__float2int_rn(dt * v * t.k.isy);
+    return b;
+}
+__device__ __forceinline__ A64 moved(const A64 &a, const TruthArgs &t, bool walls, double u, double v)
+{
+    A64 b = a;
+    b.x = a.x + t.dt * u;
+    b.y = a.y + t.dt * v;
+    if (walls) b.x = fmin(fmax(b.x, 0.0), t.g.Lx);
+    else if (!(b.x >= 0.0 && b.x < t.g.Lx)) b.x -= t.g.Lx * floor(b.x / t.g.Lx);
+    if (!(b.y >= 0.0 && b.y < t.g.Ly)) b.y -= t.g.Ly * floor(b.y / t.g.Ly);
+    return b;
+}
+
+// exclusive scan of one value per thread over the block; total to all threads
+__device__ __forceinline__ int block_excl(int v, int *ws, int &total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) ws[warp] = x;
+    __syncthreads();
+    int base = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < TT / 32; w++) {
+        base += w < warp ? ws[w] : 0;
+        total += ws[w];
+    }
+    return base + x - v;
+}
+
+template <class T>
+__global__ void __launch_bounds__(TT)
+k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, TruthArgs a, TruthBins tb, Work<T> w,
+            int nsteps)
+{
+    using R = typename T::R;
+    using A = typename T::A;
+    cg::grid_group grid = cg::this_grid();
+    __shared__ int ws[TT / 32];
+    __shared__ float wmax[TT / 32], wsum[TT / 32];
+    const long long n = a.n, gt = blockIdx.x * (long long)TT + threadIdx.x, gs = gridDim.x * (long long)TT;
+    const bool walls = a.g.walls != 0;
+    const int nbins = tb.nbins(), nb1 = tb.nbx * tb.nby;
+    const float sx = a.k.sx, sy = a.k.sy, Lx = (float)a.g.Lx, Ly = (float)a.g.Ly;
+    R *fd = reinterpret_cast<R *>(a.fd);
+    unsigned long long ndeep = 0;
+    bool bad = false;
+
+    // a sum of the floes' speeds over the grid into ctl[at]; the order of its
+    // additions varies, and with it the skins, but no result
+    auto add_speeds = [&](float vs, int at) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) vs += __shfl_xor_sync(0xffffffffu, vs, d);
+        if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = vs;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int i = 1; i < TT / 32; i++) vs += wsum[i];
+            atomicAdd(reinterpret_cast<float *>(&w.ctl[at]), vs);
+        }
+    };
+    float vs0 = 0.0f;
+    for (long long l = gt; l < n; l += gs) {
+        w.A[0][l] = load_a(in, l);
+        w.B[0][l] = {in.u[l], in.v[l], in.w[l], in.th[l]};
+        vs0 += hypotf((float)in.u[l], (float)in.v[l]);
+    }
+    for (long long i = gt; i < nbins; i += gs) tb.count[i] = 0;
+    for (long long i = gt; i < nsteps; i += gs) {
+        R ua, va;
+        wind_at(P, (double)(a.step + i) * a.dt, ua, va);
+        w.wind[i] = make_double2((double)ua, (double)va);
+    }
+    if (gt < 3) w.ctl[gt] = gt == 2 ? 1 : 0;      // step -1 asks step 0 for lists
+    if (gt >= 3 && gt < 7) w.ctl[gt] = 0;
+    grid.sync();
+    add_speeds(vs0, 5 + 1);       // for the first build
+    grid.sync();
+
+    int cur = 0, par = 0;
+    for (int s = 0; s < nsteps; s++) {
+        const bool need = *(volatile int *)&w.ctl[(s + 2) % 3] != 0;
+        if (gt == 0) w.ctl[(s + 1) % 3] = 0;      // read at the last step, written at the next
+        if (need) {
+            // count the floes of each bin; skins: 48 steps' way at the current speed,
+            // or at half the mean one (at the build before), plus 2 % of the radius
+            float smax = 0.0f, vsum = 0.0f;
+            const float vfloor = 0.5f * __int_as_float(*(volatile int *)&w.ctl[5 + (par ^ 1)]) / (float)n;
+            for (long long l = gt; l < n; l += gs) {
+                const A p = w.A[cur][l];
+                const Rest<R> q = w.B[cur][l];
+                const uint2 x = fixed(p, a.g);
+                const float u = (float)q.u, v = (float)q.v, r = (float)p.r;
+                const float speed = sqrtf(u * u + v * v);
+                vsum += speed;
+                const float skin = 48.0f * (float)a.dt * fmaxf(speed, vfloor) + 0.02f * r;
+                w.skin[l] = skin;
+                w.xb[l] = x;
+                smax = fmaxf(smax, skin);
+                const int b = r <= tb.r_split ? fbin(x.y, tb.nby) * tb.nbx + fbin(x.x, tb.nbx)
+                                              : nb1 + fbin(x.y, tb.nby2) * tb.nbx2 + fbin(x.x, tb.nbx2);
+                w.binof[l] = b;
+                w.rank[l] = atomicAdd(&tb.count[b], 1);
+            }
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, d));
+            if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = smax;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int i = 1; i < TT / 32; i++) smax = fmaxf(smax, wmax[i]);
+                atomicMax(&w.ctl[3 + par], __float_as_int(smax));   // skins are positive: ordered as integers
+            }
+            add_speeds(vsum, 5 + par);
+            grid.sync();
+            // each block a run of bins: its total, then the starts
+            const int per = (nbins + gridDim.x - 1) / gridDim.x;
+            const int c0 = min((int)blockIdx.x * per, nbins), c1 = min(c0 + per, nbins);
+            const int each = (per + TT - 1) / TT;
+            const int t0 = min(c0 + (int)threadIdx.x * each, c1), t1 = min(t0 + each, c1);
+            int sum = 0;
+            for (int i = t0; i < t1; i++) sum += tb.count[i];
+            int total;
+            const int mine = block_excl(sum, ws, total);
+            if (threadIdx.x == 0) w.bsum[blockIdx.x] = total;
+            if (gt == 0) w.ctl[3 + (par ^ 1)] = w.ctl[5 + (par ^ 1)] = 0;   // the next build's sums
+            grid.sync();
+            int before = 0;
+            for (int i = threadIdx.x; i < (int)blockIdx.x; i += TT) before += w.bsum[i];
+            block_excl(before, ws, before);
+            int run = before + mine;
+            for (int i = t0; i < t1; i++) {
+                tb.start[i] = run;
+                run += tb.count[i];
+                tb.count[i] = 0;
+            }
+            grid.sync();
+            for (long long l = gt; l < n; l += gs) {
+                const uint2 x = w.xb[l];
+                // the reach covers the rounding of the FP32 tests
+                const float reach = ((float)w.A[cur][l].r + w.skin[l]) * 1.00001f + 1.0e-9f * fmaxf(Lx, Ly);
+                w.sorted[tb.start[w.binof[l]] + w.rank[l]] = {x.x, x.y, reach, (int)l};
+            }
+            grid.sync();
+        }
+        // the largest skin of the lists in use (of either parity's build)
+        if (need) par ^= 1;
+        const float smax = __int_as_float(*(volatile int *)&w.ctl[3 + (par ^ 1)]);
+        // f(floe, fixed-point x, y, reach) over the floes that floe l at build
+        // position x with its own reach may touch
+        auto near = [&](uint2 x, float own, auto &&f) {
+            auto range = [&](int i0, int i1) {
+                for (int i = i0; i < i1; i++) {
+                    const Sorted q = w.sorted[i];
+                    const float dx = sep_x(q.x, x.x, sx, walls), dy = (float)(int)(q.y - x.y) * sy, r = own + q.reach;
+                    if (!(dx * dx + dy * dy >= r * r)) f(q.l);   // NaN passes
+                }
+            };
+            const float r1 = own + (tb.r_split + smax) * 1.00001f, r2 = own + (tb.r_max + smax) * 1.00001f;
+            visit_ranges(tb.start, 0, tb.nbx, tb.nby, x, r1 * tb.nbx / Lx, r1 * tb.nby / Ly, walls, range);
+            if (tb.nbx2 > 0)
+                visit_ranges(tb.start, nb1, tb.nbx2, tb.nby2, x, r2 * tb.nbx2 / Lx, r2 * tb.nby2 / Ly, walls, range);
+        };
+        auto own_reach = [&](long long l, R r) { return ((float)r + w.skin[l]) * 1.00001f + 1.0e-9f * fmaxf(Lx, Ly); };
+        if (need) {
+            for (long long l = gt; l < n; l += gs) {
+                int c = 0;
+                near(w.xb[l], own_reach(l, w.A[cur][l].r), [&](int j) {
+                    if (j == (int)l) return;
+                    if (c < LT) w.list[c * n + l] = j;
+                    c++;
+                });
+                w.cnt[l] = c;
+                if (c > 1 && c <= 16) sort_list<16>(w.list + l, n, c);
+                else if (c > 16 && c <= LT) sort_list<LT>(w.list + l, n, c);
+            }
+        }
+        const bool last = s == nsteps - 1;
+        const double2 wa = w.wind[s];
+        bool far = false;
+        for (long long l = gt; l < n; l += gs) {
+            const A me = w.A[cur][l];
+            const Rest<R> q = w.B[cur][l];
+            R fx = 0, fy = 0, tq = 0;
+            unsigned deep = 0;
+            auto contact = [&](int j, const A &o) {
+                R dx, dy;
+                pair_xy(o, me, a, walls, dx, dy);
+                const R d2 = dx * dx + dy * dy, S = me.r + o.r;
+                if (d2 < S * S) {
+                    const Rest<R> p = w.B[cur][j];
+                    contact_add(dx, dy, d2, me.r, o.r, me.h, o.h, p.u - q.u, p.v - q.v, q.w, p.w, P, fx, fy, tq, deep);
+                }
+            };
+            const int c = w.cnt[l];
+            if (c <= LT) {
+                for (int i = 0; i < c; i += 4) {      // four partners' loads in flight
+                    int j[4];
+                    A o[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) j[k] = w.list[min(i + k, c - 1) * n + l];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) o[k] = w.A[cur][j[k]];
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        if (i + k < c) contact(j[k], o[k]);
+                }
+            } else {
+                // more candidates than a list holds: the smallest partner above the
+                // last one, until there is none
+                const uint2 x = w.xb[l];
+                const float own = own_reach(l, me.r);
+                for (int lastj = -1;;) {
+                    int best = INT_MAX;
+                    near(x, own, [&](int j) {
+                        if (j <= lastj || j >= best || j == (int)l) return;
+                        R dx, dy;
+                        const A o = w.A[cur][j];
+                        pair_xy(o, me, a, walls, dx, dy);
+                        const R S = me.r + o.r;
+                        if (dx * dx + dy * dy < S * S) best = j;
+                    });
+                    if (best == INT_MAX) break;
+                    contact(best, w.A[cur][best]);
+                    lastj = best;
+                }
+            }
+            R uo, vo, zeta;
+            ocean_at(P, w, a, me, uo, vo, zeta);
+            if (walls) wall_force(me, a, q.u, q.v, q.w, P, fx, fy, tq, deep);
+            R Fdx, Fdy, Td;
+            drag_force(P, uo, vo, zeta, (R)wa.x, (R)wa.y, q.u, q.v, q.w, me.r, Fdx, Fdy, Td);
+            fx += Fdx; fy += Fdy; tq += Td;
+            const R dt = (R)a.dt;
+            const R m = P.mass_c * me.r * me.r * me.h;
+            const R I = P.inertia_f * m * me.r * me.r;
+            const A to = moved(me, a, walls, q.u, q.v);
+            const Rest<R> v = {q.u + dt * (fx / m), q.v + dt * (fy / m), q.w + dt * (tq / I), q.th + dt * q.w};
+            bad |= !(isfinite(v.u) && isfinite(v.v) && isfinite(v.w));
+            ndeep += deep ? 1u : 0u;
+            if (last) {
+                store_xy(out, l, to);
+                out.u[l] = v.u;
+                out.v[l] = v.v;
+                out.w[l] = v.w;
+                out.th[l] = v.th;
+                out.r[l] = me.r;
+                out.h[l] = me.h;
+                fd[l] = Fdx; fd[n + l] = Fdy; fd[2 * n + l] = Td;
+            } else {
+                w.A[cur ^ 1][l] = to;
+                w.B[cur ^ 1][l] = v;
+                const uint2 x = fixed(to, a.g), x0 = w.xb[l];
+                const float bx = sep_x(x.x, x0.x, sx, walls), by = (float)(int)(x.y - x0.y) * sy, sk = w.skin[l];
+                far |= !(bx * bx + by * by <= sk * sk);
+            }
+        }
+        if (last) break;
+        if (__syncthreads_or(far) && threadIdx.x == 0) w.ctl[s % 3] = 1;
+        grid.sync();
+        cur ^= 1;
+    }
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&a.ctrl->err, ERR_NONFINITE);
+    if (ndeep) atomicAdd(&a.ctrl->deep, ndeep);
+}
+
+template <class T>
+int grid_of(long long n)
+{
+    static int per_sm = 0, nsm = 0;
+    if (!per_sm) {
+        int dev = 0, b = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_truth_run<T>, TT, 0) != cudaSuccess) b = 0;
+        per_sm = b > 0 ? b : 1;
+    }
+    const long long need = (n + TT - 1) / TT, most = (long long)per_sm * nsm;
+    return (int)(need < 1 ? 1 : (need < most ? need : most));
+}
+
+// the work arrays in one allocation of `bytes` (base NULL: only its size)
+template <class T>
+Work<T> carve(unsigned char *base, long long n, const Phys<double> &P, const Geom &g, size_t &bytes)
+{
+    size_t o = 0;
+    auto take = [&](auto *&p, size_t count) {
+        using E = std::remove_reference_t<decltype(*p)>;
+        p = reinterpret_cast<E *>(base + o);
+        o += (sizeof(E) * count + 255) & ~size_t(255);
+    };
+    Work<T> w{};
+    const bool wide = sizeof(typename T::R) == 8;
+    for (int k = 0; k < 2; k++) {
+        take(w.A[k], n);
+        take(w.B[k], n);
+    }
+    take(w.binof, n);
+    take(w.rank, n);
+    take(w.cnt, n);
+    take(w.list, (size_t)LT * n);
+    take(w.xb, n);
+    take(w.skin, n);
+    take(w.sorted, n);
+    take(w.bsum, 4096);
+    take(w.ctl, 8);
+    take(w.wind, TRUTH_CHUNK);
+    if (wide) tile_counts(P, g, w.tx, w.ty);
+    take(w.tile, (size_t)w.tx * w.ty * P.n_modes);
+    bytes = o;
+    return w;
+}
+
+template <class T>
+cudaError_t launch(const typename T::State &in, const typename T::State &out, const Phys<typename T::R> &P,
+                   const Phys<double> &P64, const TruthArgs &a, TruthBins &b, void *work, int nsteps, cudaStream_t st)
+{
+    if (a.n <= 0 || nsteps <= 0) return cudaSuccess;
+    size_t bytes;
+    Work<T> w = carve<T>(static_cast<unsigned char *>(work), a.n, P64, a.g, bytes);
+    typename T::State si = in, so = out;
+    Phys<typename T::R> p = P;
+    TruthArgs ta = a;
+    void *args[] = {&si, &so, &p, &ta, &b, &w, &nsteps};
+    return cudaLaunchCooperativeKernel((const void *)k_truth_run<T>, dim3(grid_of<T>(a.n)), dim3(TT), args, 0, st);
+}
+
+}  // namespace
+
+size_t truth_work_bytes(int precision, long long n, const Phys<double> &P, const Geom &g)
+{
+    size_t bytes = 0;
+    if (precision == 1) carve<Tr64>(nullptr, n, P, g, bytes);
+    else carve<Tr32>(nullptr, n, P, g, bytes);
+    return bytes;
+}
+
+cudaError_t truth_work_init(int precision, long long n, const Phys<double> &P, const Geom &g, void *work, cudaStream_t st)
+{
+    if (precision != 1) return cudaSuccess;
+    size_t bytes;
+    const Work<Tr64> w = carve<Tr64>(static_cast<unsigned char *>(work), n, P, g, bytes);
+    const int k = w.tx * w.ty * P.n_modes;
+    if (k > 0) k_truth_tiles<<<(k + 255) / 256, 256, 0, st>>>(P, g, w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_truth_run32(const DevState32 &in, const DevState32 &out, const Phys<float> &P, const Phys<double> &P64,
+                               const TruthArgs &a, TruthBins &b, void *work, int nsteps, cudaStream_t st)
+{
+    return launch<Tr32>(in, out, P, P64, a, b, work, nsteps, st);
+}
+
+cudaError_t launch_truth_run64(const DevState64 &in, const DevState64 &out, const Phys<double> &P, const TruthArgs &a,
+                               TruthBins &b, void *work, int nsteps, cudaStream_t st)
+{
+    return launch<Tr64>(in, out, P, P, a, b, work, nsteps, st);
+}
+
+}  // namespace msd
