@@ -481,11 +481,17 @@ static StepCommon cell_common(ms_model *m, long long i_local, bool scratch_out)
     return sc;
 }
 
-// the cell kernels of a run of steps inside one coarse interval (FP32
-// variants 2-5): every size class's steps on its own stream, forked once
+// FP64 cells stay in shared memory for a run of steps unless one is too large
+static bool resident64(const ms_model *m) { return m->precision == MS_FP64 && m->max_n <= RUN64_MAX; }
+
+// the cell kernels of a run of steps inside one coarse interval: FP64, one
+// launch; FP32 variants 2-5, every size class's steps on its own stream,
+// forked once
 static cudaError_t launch_run_cells(ms_model *m, long long i_local, int nsteps, bool scratch_out)
 {
     const StepCommon sc = cell_common(m, i_local, scratch_out);
+    if (resident64(m))
+        return launch_cell_run64(m->s64, scratch_out ? m->x64 : m->s64, m->P64, sc, m->cl, nsteps, m->stream);
     cudaError_t e = cell_fork(m->cl, m->stream);
     if (e == cudaSuccess) e = launch_cell_run32(m->s32, scratch_out ? m->x32 : m->s32, m->P32, sc, m->cl, nsteps);
     if (e == cudaSuccess) e = cell_join(m->cl, m->stream);
@@ -498,11 +504,15 @@ static cudaError_t launch_interval_cells(ms_model *m, bool scratch_out)
     return launch_run_cells(m, 0, m->interval, scratch_out);
 }
 
-static bool interval_cells(const ms_model *m) { return m->precision == MS_FP32 && m->cl.variant >= 2; }
+static bool interval_cells(const ms_model *m)
+{
+    return resident64(m) || (m->precision == MS_FP32 && m->cl.variant >= 2);
+}
 
 // cell-kernel launches of one coarse interval on the graph path
 static int64_t interval_launches(const ms_model *m)
 {
+    if (resident64(m)) return 1;
     if (m->cl.variant == 0 || m->precision == MS_FP64) return m->interval;
     int64_t k = 0;
     for (int s = 0; s < m->cl.nseg; s++)
@@ -512,6 +522,7 @@ static int64_t interval_launches(const ms_model *m)
 
 static cudaError_t launch_step(ms_model *m, long long i_local, bool scratch_out)
 {
+    if (resident64(m)) return launch_run_cells(m, i_local, 1, scratch_out);
     StepCommon sc = cell_common(m, i_local, scratch_out);
     if (m->precision == MS_FP64)
         return launch_cell_step64(m->s64, scratch_out ? m->x64 : m->s64, m->P64, sc, m->cl, m->stream);
@@ -1575,9 +1586,9 @@ static int step_enqueue(ms_model *m, double dt, int64_t nsteps)
             CK(launch_interval_start(m));
         }
         // What is left of the call or of the interval, whichever ends first.
-        // The FP32 size classes take it as one run: a launch per fine step
-        // would load the floes, build the candidate lists and reduce the
-        // moments at every step.
+        // The resident cells and the FP32 size classes take it as one run: a
+        // launch per fine step would load the floes, build the candidate
+        // lists and reduce the moments at every step.
         const long long run = interval_cells(m) ? std::min<long long>(nsteps, N - i_local) : 1;
         {
             Trace tf("msdem.fine step");

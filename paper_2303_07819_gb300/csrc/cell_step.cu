@@ -2361,7 +2361,7 @@ cudaError_t cell_step_prepare(int, const CellLaunch &, size_t smem)
             (const void *)k_cell_step32_wlist<4>, (const void *)k_cell_step32_binned<64, true>,
             (const void *)k_cell_step32_binned<128, true>, (const void *)k_cell_step32_binned<256, true>};
         limit = optin;
-        if ((e = run_block_prepare()) != cudaSuccess) return e;
+        if ((e = run_block_prepare()) != cudaSuccess || (e = run64_prepare()) != cudaSuccess) return e;
         for (const void *k : kern) {
             cudaFuncAttributes fa;
             e = cudaFuncGetAttributes(&fa, k);

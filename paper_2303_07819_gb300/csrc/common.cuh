@@ -87,10 +87,29 @@ struct Geom {
 template <class R> __device__ __forceinline__ R dmin(R a, R b) { return a < b ? a : b; }
 template <class R> __device__ __forceinline__ R dmax(R a, R b) { return a > b ? a : b; }
 
-// 1/sqrt(x): the hardware reciprocal square root in FP32, the IEEE
-// operations in FP64 (the parity path)
-__device__ __forceinline__ float inv_sqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
+// 1/sqrt(x) of a square of lengths or speeds: the hardware reciprocal square
+// root in FP32 (within 2 ulp), rsqrt in FP64 (within 1 ulp; the parity path).
+// Arguments below the smallest normal number count as it, which spares the
+// scaling of subnormal arguments around rsqrtf and keeps 0 finite: two such
+// norms per floe-step cost 47 of its 400 instructions with rsqrtf, 10 so.
+__device__ __forceinline__ float inv_sqrt(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(x, 1.17549435e-38f)));
+    return y;
+}
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+
+// sqrt(x): in FP32 one Newton step s + (x - s^2) / (2 sqrt(x)) from s = x
+// rsqrt(x), the residual exact in an FMA; x below the smallest normal number
+// counts as it (a contact at onset, where d rounds to r_l + r_j or above,
+// asks for the root of 0 or of a little less)
+__device__ __forceinline__ float root(float x)
+{
+    const float p = fmaxf(x, 1.17549435e-38f), y = inv_sqrt(p), s = __fmul_rn(p, y);
+    return __fmaf_rn(__fmaf_rn(-s, s, p), __fmul_rn(0.5f, y), s);
+}
+__device__ __forceinline__ double root(double x) { return sqrt(x); }
 
 // Contact of floe l with floe j given the minimum-image separation
 // (dx, dy) = x_j - x_l.  Eq. (2.2): n from l to j, delta = d - (r_l + r_j) < 0
@@ -101,7 +120,35 @@ __device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
 // c^2 d^2 = (S - d)(S + d)(d - D)(d + D), S = r_l + r_j, D = r_l - r_j
 // (Heron's formula for the triangle (d, r_l, r_j)); a floe inside the other
 // (d <= |D|) gives the smaller diameter.
-// Returns true on contact and adds the force on l to (fx, fy, tq).
+// contact_force: the force (gx, gy) on l and the tangential part ft (torque
+// r_l ft) of a pair in contact (0 < d2 < (r_l + r_j)^2).
+template <class R>
+__device__ __forceinline__ void contact_force(R dx, R dy, R d2, R rl, R rj, R hl, R hj,
+                                              R dux, R duy, R wl, R wj, const Phys<R> &P,
+                                              R &gx, R &gy, R &ft, unsigned &deep)
+{
+    const R S = rl + rj;
+    const R id = inv_sqrt(d2);
+    const R d = d2 * id;
+    const R nx = dx * id, ny = dy * id;
+    const R delta = d - S;
+    const R D = rl - rj;
+    const R Q = (d - D) * (d + D);
+    const R c = (Q <= R(0)) ? R(2) * dmin(rl, rj) : root((-delta) * (S + d) * Q) * id;
+    const R hc = dmin(hl, hj) * P.inv_h_ref;
+    const R vn = dux * nx + duy * ny;
+    R Fn = c * hc * (P.E * delta + P.eta * vn);
+    Fn = dmin(Fn, R(0));
+    const R vt = dux * (-ny) + duy * nx - wj * rj - wl * rl;
+    ft = c * hc * P.G * vt;
+    const R cap = P.mu * (-Fn);
+    ft = dmax(dmin(ft, cap), -cap);
+    gx = Fn * nx - ft * ny;
+    gy = Fn * ny + ft * nx;
+    deep |= (delta < R(-0.5) * dmin(rl, rj)) ? 1u : 0u;
+}
+
+// contact_add returns true on contact and adds the force on l to (fx, fy, tq).
 template <class R>
 __device__ __forceinline__ bool contact_add(R dx, R dy, R d2, R rl, R rj, R hl, R hj,
                                             R dux, R duy, R wl, R wj, const Phys<R> &P,
@@ -109,25 +156,11 @@ __device__ __forceinline__ bool contact_add(R dx, R dy, R d2, R rl, R rj, R hl, 
 {
     const R S = rl + rj;
     if (!(d2 > R(0) && d2 < S * S)) return false;
-    const R id = inv_sqrt(d2);
-    const R d = d2 * id;
-    const R nx = dx * id, ny = dy * id;
-    const R delta = d - S;
-    const R D = rl - rj;
-    const R Q = (d - D) * (d + D);
-    const R c = (Q <= R(0)) ? R(2) * dmin(rl, rj) : sqrt((-delta) * (S + d) * Q) * id;
-    const R hc = dmin(hl, hj) * P.inv_h_ref;
-    const R vn = dux * nx + duy * ny;
-    R Fn = c * hc * (P.E * delta + P.eta * vn);
-    Fn = dmin(Fn, R(0));
-    const R vt = dux * (-ny) + duy * nx - wj * rj - wl * rl;
-    R ft = c * hc * P.G * vt;
-    const R cap = P.mu * (-Fn);
-    ft = dmax(dmin(ft, cap), -cap);
-    fx += Fn * nx - ft * ny;
-    fy += Fn * ny + ft * nx;
+    R gx, gy, ft;
+    contact_force(dx, dy, d2, rl, rj, hl, hj, dux, duy, wl, wj, P, gx, gy, ft, deep);
+    fx += gx;
+    fy += gy;
     tq += rl * ft;
-    deep |= (delta < R(-0.5) * dmin(rl, rj)) ? 1u : 0u;
     return true;
 }
 
@@ -399,6 +432,12 @@ cudaError_t cell_fork(const CellLaunch &cl, cudaStream_t st);
 cudaError_t cell_join(const CellLaunch &cl, cudaStream_t st);
 cudaError_t launch_cell_step64(const DevState64 &in, const DevState64 &out, const Phys<double> &P,
                                const StepCommon &sc, const CellLaunch &cl, cudaStream_t st);
+// cell_run64.cu: nsteps fine steps from step sc.i_local of the interval, every
+// cell in its block's shared memory; cells of at most RUN64_MAX floes
+constexpr int RUN64_MAX = 1024;
+cudaError_t launch_cell_run64(const DevState64 &in, const DevState64 &out, const Phys<double> &P,
+                              const StepCommon &sc, const CellLaunch &cl, int nsteps, cudaStream_t st);
+cudaError_t run64_prepare();
 cudaError_t launch_cell_moments32(const DevState32 &s, const Phys<float> &P, const StepCommon &sc,
                                   cudaStream_t st);
 cudaError_t launch_cell_moments64(const DevState64 &s, const Phys<double> &P, const StepCommon &sc,
