@@ -12,6 +12,9 @@
 #include <thread>
 #include <vector>
 
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include <nvtx3/nvToolsExt.h>
 
 #include "classes.cuh"
@@ -248,6 +251,47 @@ static void host_parallel(long long n, F &&f)
     }
     f(0LL, std::min(n, chunk));
     for (auto &x : th) x.join();
+}
+
+// Make the pages of a caller's output array resident before the device writes
+// them: a copy into fresh pageable memory takes the device a fault a page
+// (25 MB of moments: 4.4 ms more than into resident pages), which the host's
+// cores serve sooner, and while the device still computes what is to be copied.
+static void host_pages(void *p, size_t bytes)
+{
+    cudaPointerAttributes at;
+    if (bytes < (1u << 18)) return;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (at.type != cudaMemoryTypeUnregistered) return;
+    const size_t pg = (size_t)sysconf(_SC_PAGESIZE);
+    const uintptr_t b0 = (uintptr_t)p, lo = b0 / pg * pg, np = (b0 + bytes - lo + pg - 1) / pg;
+    try {
+        std::vector<unsigned char> in(np);
+        if (mincore((void *)lo, np * pg, in.data()) != 0) return;
+        size_t gone = 0;
+        for (unsigned char x : in) gone += !(x & 1);
+        std::atomic<size_t> next{0};
+        auto touch = [&] {
+            for (size_t i; (i = next.fetch_add(1)) < np;)
+                if (!(in[i] & 1)) {
+                    volatile unsigned char *q = (volatile unsigned char *)std::max(b0, lo + i * pg);
+                    *q = *q;
+                }
+        };
+        const size_t nt = std::min<size_t>({8, gone * pg >> 20, std::thread::hardware_concurrency()});
+        std::vector<std::thread> th;
+        th.reserve(8);
+        try {
+            for (size_t t = 1; t < nt; t++) th.emplace_back(touch);
+        } catch (...) {   // no further thread to be had: the others take its share
+        }
+        if (gone) touch();
+        for (auto &x : th) x.join();
+    } catch (...) {       // no memory for the list: the device takes the faults
+    }
 }
 
 // smallest index in [0, n) for which bad(l) holds, or n
@@ -1614,6 +1658,7 @@ static int step_enqueue(ms_model *m, double dt, int64_t nsteps)
 int ms_moments(ms_model *m, double *out)
 {
     if (!m || !out) return fail(MS_ERR_ARG, "NULL argument");
+    host_pages(out, sizeof(double) * m->ncell * NMOM);
     CK(cudaMemcpyAsync(out, m->d_mom, sizeof(double) * m->ncell * NMOM, cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
     return MS_OK;
@@ -1649,6 +1694,7 @@ static int download(ms_model *m, bool truth, double *out)
         CK(launch_cells_to_floes64(truth ? m->t64[m->tcur] : m->s64, orig, m->d_cell_of, g, m->d_raw, m->stream));
     else
         CK(launch_cells_to_floes32(truth ? m->t32[m->tcur] : m->s32, orig, m->d_cell_of, g, m->d_raw, m->stream));
+    host_pages(out, sizeof(double) * 8 * m->n);
     CK(cudaMemcpyAsync(out, m->d_raw, sizeof(double) * 8 * m->n, cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
     return MS_OK;
@@ -1759,6 +1805,7 @@ int ms_truth_moments(ms_model *m, double *out)
     const TruthArgs a = truth_args(m, m->truth_dt > 0 ? m->truth_dt : 1.0, m->truth_steps);
     if (m->precision == MS_FP64) CK(launch_truth_moments64(m->t64[m->tcur], m->P64, a, m->cb, m->d_tmom, m->stream));
     else CK(launch_truth_moments32(m->t32[m->tcur], m->P32, a, m->cb, m->d_tmom, m->stream));
+    host_pages(out, sizeof(double) * m->ncell * NMOM);
     CK(cudaMemcpyAsync(out, m->d_tmom, sizeof(double) * m->ncell * NMOM, cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
     return MS_OK;
