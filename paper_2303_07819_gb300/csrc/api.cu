@@ -447,6 +447,8 @@ static Geo32 geo32(double Lx, double Ly, int nx, int ny, double dt)
     k.iLx = (float)(1.0 / Lx);
     k.iLy = (float)(1.0 / Ly);
     k.dt = (float)dt;
+    k.dtsx = k.dt * k.isx;
+    k.dtsy = k.dt * k.isy;
     return k;
 }
 
@@ -475,6 +477,7 @@ static StepCommon step_common(ms_model *m, long long i_local, double *mom, doubl
     sc.carry_in = m->d_carry;
     sc.carry_out = m->d_carry;
     sc.ncarry = m->n;
+    sc.fresh = 0;
     return sc;
 }
 
@@ -533,7 +536,8 @@ static bool resident64(const ms_model *m) { return m->precision == MS_FP64 && m-
 // forked once
 static cudaError_t launch_run_cells(ms_model *m, long long i_local, int nsteps, bool scratch_out)
 {
-    const StepCommon sc = cell_common(m, i_local, scratch_out);
+    StepCommon sc = cell_common(m, i_local, scratch_out);
+    sc.fresh = !sc.couple && nsteps < m->interval;
     if (resident64(m))
         return launch_cell_run64(m->s64, scratch_out ? m->x64 : m->s64, m->P64, sc, m->cl, nsteps, m->stream);
     cudaError_t e = cell_fork(m->cl, m->stream);

@@ -318,6 +318,7 @@ struct Geo32 {
     float Lx, Ly;       // cell sides (m)
     float iLx, iLy;
     float dt;
+    float dtsx, dtsy;   // dt isx, dt isy
 };
 
 // Contact candidate lists of the FP32 state (variant 4): per floe up to NBL
@@ -365,6 +366,8 @@ struct StepCommon {
     const float *carry_in;
     float *carry_out;
     long long ncarry;
+    int fresh;          // variant 5, a run whose floes' centres nobody picks up (uncoupled, shorter than the
+                        // interval): every step takes new ones, so that it gives the same however it is split
 };
 
 // 2^32 and 2^-32: fixed-point positions of the FP32 path (2^32 = cell side)
@@ -403,8 +406,8 @@ constexpr int RUN_T = 256;      // threads per block of the resident block kerne
 constexpr int RUN_GCMAX = 32;   // cells per group of those kernels
 constexpr int RUN_NCARRY = 7;   // words per floe a run hands to the next: 5 window sums, ocean expansion centre
 
-// cell_run.cu: a run of nsteps fine steps of one block class (K floes per
-// thread) from step sc.i_local of the interval, every floe in registers
+// cell_run.cu: a run of nsteps fine steps of one block class (blocks of K
+// RUN_T floes) from step sc.i_local of the interval, every floe in registers
 // (launch variant 5).  groups[g] = (first slot, cells, floes, bins incl. one
 // large-floe slot per cell) in processing order; items[slot] = (cell, first
 // floe of the cell in its group, bins per side (0: none), bin base); the

@@ -1,6 +1,7 @@
-"""The resident FP64 cells and the truth DEM's lists against the oracle, at the
-sizes where their branches part.  Tolerances as in the parity tests: 1e-10
-(FP64) and 1e-4 (FP32), relative, per moment column."""
+"""The resident FP64 cells, the long candidate lists of the resident FP32 cells
+and the truth DEM's lists against the oracle, at the sizes where their
+branches part.  Tolerances as in the parity tests: 1e-10 (FP64) and 1e-4
+(FP32), relative, per moment column."""
 import numpy as np
 import pytest
 
@@ -77,6 +78,52 @@ def test_fp64_cells(orc, ms, n, threads, persistent):
     fa, fb = a.floes(), b.floes()
     assert all(np.array_equal(fa[k], fb[k]) for k in fa)
     assert np.array_equal(a.coupling()["window"], b.coupling()["window"])
+
+
+@pytest.mark.parametrize("n,big,small", [(11, 3000.0, 400.0), (13, 3000.0, 400.0), (24, 4000.0, 400.0), (26, 4000.0, 400.0),
+                                         (200, 5000.0, 150.0), (300, 5000.0, 150.0), (600, 5000.0, 100.0)])
+def test_fp32_long_lists(orc, ms, n, big, small):
+    """A large floe with n partners: lists up to the slots of a build's first
+    sort, beyond them, and long enough for a whole warp to walk."""
+    side = 25e3
+    f, p = ring(n, side, big, small), soft(1, side)
+    o, g = orc.Model(p, f), ms.Model(p, f, ms.MS_FP32)
+    o.step(10.0, 23)
+    g.step(10.0, 23)
+    e = rel_errors(g.moments(), o.moments(), p, TOL[0][1])
+    assert e.max() <= TOL[0][0], report(e)
+
+
+@pytest.mark.parametrize("n", [40, 250, 500, 900])
+def test_fp32_lists_that_do_not_fit(orc, ms, n):
+    """So crowded that a group's lists exceed their room: every pair of the
+    cell is tested."""
+    side = 25e3
+    f, p = crowd(n, n, side, 5.0), soft(1, side)
+    o, g = orc.Model(p, f), ms.Model(p, f, ms.MS_FP32)
+    o.step(10.0, 12)
+    g.step(10.0, 12)
+    e = rel_errors(g.moments(), o.moments(), p, TOL[0][1])
+    assert e.max() <= TOL[0][0], report(e)
+
+
+@pytest.mark.parametrize("nx,n", [(1, 400), (3, 30), (6, 3)])
+def test_fp32_uncoupled_split(ms, nx, n):
+    """Uncoupled steps short of a whole interval give the same floes however
+    they are split into calls, to the last bit."""
+    side = 25e3
+    parts = [crowd(c, n, side, 0.7) for c in range(nx * nx)]
+    for c, f in enumerate(parts):
+        f["x"] += side * (c % nx)
+        f["y"] += side * (c // nx)
+    f, p = join(parts), dict(soft(nx, nx * side), couple=0)
+    a, b = ms.Model(p, f, ms.MS_FP32), ms.Model(p, f, ms.MS_FP32)
+    a.step(10.0, 61)
+    for k in (1, 1, 7, 33, 19):
+        b.step(10.0, k)
+    fa, fb = a.floes(), b.floes()
+    assert all(np.array_equal(fa[k], fb[k]) for k in fa)
+    assert np.array_equal(a.moments(), b.moments())
 
 
 @pytest.mark.parametrize("precision", [0, 1])
