@@ -227,8 +227,8 @@ int ms_autotune(ms_model *m, double dt, int32_t reps, double *best_ms);
  * larger ones block-per-cell; variant 5 (the default) keeps every cell of up
  * to 1024 floes resident in registers for a whole run of steps (one launch
  * per coarse interval on the graph path): a floe per thread of a 256-thread
- * block that several small cells share, 2 or 4 floes per thread for cells of
- * 257-512 or 513-1024 floes, blocks taking groups of cells from a work queue
+ * block that several small cells share, or of a block of 512 or 1024 threads
+ * for a cell of 257-512 or 513-1024 floes, blocks taking groups of cells from a work queue
  * largest first; contact candidates from per-floe skins, summed in
  * ascending partner order; larger cells run the block list kernel step by
  * step (see ms_set_resident for its tunables).  Variants 2-5 give the same
@@ -250,7 +250,8 @@ int ms_time_kernel(ms_model *m, int32_t which, double dt, int32_t reps, double *
  * again -- is its speed (plus what the coming gradual updates add) times
  * skin_steps fine steps (1 .. 1000); cells of at most 256 floes share a
  * block of 256 threads, a floe per thread, up to block_floes (32 .. 256)
- * floes in all; a larger cell has a block of its own.  Floes do not depend
+ * floes in all (fewer where the model is too small to fill the SMs with such
+ * blocks); a larger cell has a block of its own.  Floes do not depend
  * on skin_steps, block_floes or the other cells of the model, and
  * neither do the moments: the per-cell sums are exact fixed-point integer
  * sums (each value relative to the largest binary exponent of its cell and

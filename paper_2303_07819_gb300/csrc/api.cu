@@ -893,11 +893,11 @@ static cudaError_t fold_carry(ms_model *m)
 }
 
 // Variant 5: the cells of the resident classes packed into the groups one
-// block takes.  A cell of more than 512 floes opens a group of 4 floes per
-// thread (1024 floes), one of more than 256 a group of 2 per thread; smaller
-// cells go, largest first, into the open group with the least room that
-// still fits them (at most RUN_GCMAX cells), else open a group of one floe
-// per thread.  Each class's groups run in decreasing order of floes.  Each
+// block takes.  A cell of more than 512 floes is a group for a block of 1024,
+// one of more than 256 for a block of 512; smaller cells go, largest first,
+// into the open group with the least room that still fits them (at most
+// RUN_GCMAX cells), else open a group for a block of RUN_T floes.  Each class's
+// groups run in decreasing order of floes.  Each
 // cell gets about sqrt(n)/beta bins per side, at most sqrt(n) (so a group's
 // bins fit its shared memory), none below 3.
 static int build_groups(ms_model *m, CellLaunch &cl)
@@ -925,10 +925,9 @@ static int build_groups(ms_model *m, CellLaunch &cl)
         g.cells.push_back(cc);
         g.nf += n;
         g.room -= n;
-        // only groups of one floe per thread take further cells: a cell's
-        // floes then run the code of its own size class wherever it is
-        // packed (the 2- and 4-floe classes compile to other instruction
-        // sequences, whose rounding may differ)
+        // only the groups of small cells take further cells: a cell's floes
+        // then run the code of its own size class wherever it is packed (the
+        // larger classes round the contact law differently)
         if (g.K == 1 && (int)g.cells.size() < RUN_GCMAX) by_room[g.room].push_back(gi);
     };
     int first_item = -1, end_item = -1;

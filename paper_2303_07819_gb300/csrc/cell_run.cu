@@ -11,13 +11,13 @@
 // cell of more than 256 or 512 floes is a group of its own, smaller cells share
 // groups of the first kind, first fit by decreasing size.  A cell's floes so
 // always run the code of its own size class, whatever else the model holds.
-// A class is one persistent launch (256 threads, 512, or 512 with two floes a
-// thread) whose blocks take groups from a ticket queue in decreasing order of
-// work.  A floe's state and forcing stay in registers for the run, what a step
-// reads once stays in shared memory (the class of 256 has 64 registers a
-// thread, four blocks an SM); per step it publishes its position and velocity
-// to shared memory (two buffers, so one barrier per step separates the step
-// that reads a buffer from the one that writes it again).
+// A class is one persistent launch of blocks of as many threads, a floe each,
+// that take groups from a ticket queue in decreasing order of work.  A floe's
+// state and forcing stay in registers for the run, what a step reads once stays
+// in shared memory (64 registers a thread, 1024 threads an SM); per step it
+// publishes its position and velocity to shared memory (two buffers, so one
+// barrier per step separates the step that reads a buffer from the one that
+// writes it again).
 //
 // What bounds it: the issue of instructions (75-80 % of the cycles on 2.0M
 // floes, no memory traffic to speak of), in steps with few floes a group the
@@ -26,8 +26,8 @@
 // a floe, a floe with more tested its whole cell; 256 threads with up to four
 // floes each; two barriers a step) and now: 65,505 power-law floes 338 -> 279
 // us fresh and 1210 -> 380 packed, 115,200 floes of one size 309 -> 264 and
-// 529 -> 455, 500,658 floes 1535 -> 1110 and 7660 -> 1460, 2.0M floes 2914 ->
-// 2850 and 3110 -> 2990, 256 floes 274 -> 190.
+// 529 -> 455, 500,658 floes 1535 -> 890 and 7660 -> 1170, 2.0M floes 2914 ->
+// 2580 and 3110 -> 2710, 256 floes 274 -> 190.
 //
 // Contacts (Eq. 2.2): a floe tests only its candidates, the floes of its
 // cell within reach at the last build: r_l G + s_l + r_j G + s_j, with G the
@@ -100,14 +100,13 @@ constexpr int GCMAX = RUN_GCMAX;   // cells per group
 constexpr int WIND = 128;          // steps per wind table
 constexpr int NRED = 16;           // values per reduction (moment columns 1-11, window sums)
 constexpr int NEVT = 16;           // gradual updates per interval with a precomputed radius ratio
-constexpr int OV_PER_K = 384;      // hits beyond a floe's LMAX slots a build holds, per floe per thread
 
 template <int RT, int K>
 struct RunSm {
     static constexpr int F = RT * K;
     static constexpr int NW = RT / 32;
     static constexpr int PAIRS = LMAX * F;      // candidate pairs of the group's lists
-    static constexpr int OV = OV_PER_K * K;
+    static constexpr int OV = F > 512 ? 768 : 384;   // hits beyond the floes' LMAX slots a build holds
     struct Buf {                    // what a floe publishes for a step
         float4 A[F];                // u, v, w, h
         uint2 Q[F];                 // fixed-point position
@@ -388,7 +387,7 @@ __device__ __forceinline__ float4 long_list_force(const RunSm<RT, K> &S, int cur
 }
 
 template <int RT, int K>
-__global__ void __launch_bounds__(RT, RT * K == RUN_T ? MS_RUN_K1_BLOCKS : 1)
+__global__ void __launch_bounds__(RT, MS_RUN_K1_BLOCKS * RUN_T / RT)
 k_cell_run32_block(DevState32 in, DevState32 out, Phys<float> P, StepCommon sc, const int4 *groups, int ngroups,
                    const int4 *items, int qslot, int nsteps, float skin_steps)
 {
@@ -1214,13 +1213,18 @@ cudaError_t launch_carry_flush(const DevState32 &s, const StepCommon &sc, float 
 }
 
 // The kernel of each class, by the floes its blocks hold in units of RUN_T:
-// f(kernel, threads, shared memory).
+// f(kernel, threads, shared memory).  A floe a thread and 64 registers in each,
+// 1024 threads an SM: the step is a chain of latencies that warps hide.  With
+// two floes a thread and half the warps the class of 256 takes 2415 us an
+// interval instead of 2044 (2.0M floes in cells of 6), and with one block an SM
+// (two floes a thread in the largest class) the larger classes 2860 instead of
+// 2560 (2.0M floes, lognormal cells) and 980 instead of 890 (500,658 floes).
 template <class F>
 static auto with_class(int K, F &&f)
 {
     if (K == 1) return f(k_cell_run32_block<RUN_T, 1>, RUN_T, sizeof(RunSm<RUN_T, 1>));
     if (K == 2) return f(k_cell_run32_block<2 * RUN_T, 1>, 2 * RUN_T, sizeof(RunSm<2 * RUN_T, 1>));
-    return f(k_cell_run32_block<2 * RUN_T, 2>, 2 * RUN_T, sizeof(RunSm<2 * RUN_T, 2>));
+    return f(k_cell_run32_block<4 * RUN_T, 1>, 4 * RUN_T, sizeof(RunSm<4 * RUN_T, 1>));
 }
 
 size_t run_block_smem(int K)

@@ -30,10 +30,10 @@ constexpr SizeClass kClassesV4[9] = {{1 << 30, 128, 0}, {640, 128, 1}, {512, 128
                                      {32, 128, 2}};
 
 // Variant 5 keeps every cell of up to 1024 floes resident for a run of
-// steps: cells of 513-1024 floes take a block of 512 threads with two floes
-// each, of 257-512 floes one of 512 threads, smaller cells share blocks of 256
-// (kind 3; the class bound in units of 256 floes names the kernel); larger
-// cells run the block-per-cell list kernel step by step.
+// steps: cells of 513-1024 floes take a block of 1024 threads, of 257-512
+// floes one of 512, smaller cells share blocks of 256 (kind 3; the class bound
+// in units of 256 floes names the kernel); larger cells run the block-per-cell
+// list kernel step by step.
 constexpr SizeClass kClassesV5[4] = {{1 << 30, 128, 0}, {1024, 256, 3}, {512, 256, 3}, {256, 256, 3}};
 
 // The streams of the first kHighPriorityClasses size classes (the largest
