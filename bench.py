@@ -584,7 +584,7 @@ def main():
                      "frac": achieved / hbm,
                      "traffic": (traffic if traffic is not None and info["variant"] == 5 else None),
                      "traffic_per": "coarse interval (one launch of each resident class)",
-                     "kernel": "msd::k_cell_run32_block<1|2|4> (resident for a coarse interval)",
+                     "kernel": "msd::k_cell_run32_block<256|512|1024> (resident for a coarse interval)",
                      "peak_source": peak_kind,
                      "bytes_per_floe_step": BYTES_PER_FLOE_STEP,
                      "algorithmic_bytes_per_interval": model.n * BYTES_PER_FLOE_STEP * N0,
