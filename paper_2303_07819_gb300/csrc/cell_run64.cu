@@ -231,6 +231,7 @@ k_cell_run64(DevState64 in, DevState64 out, Phys<double> P, StepCommon sc, int p
                     }
                     S.C[l] = (unsigned short)min(k, LM + 1);
                 }
+                __syncwarp();   // the other lanes of the warp read these lists below
             }
             RampCell rc = {1.0, 0.0, 0.0, 0.0};
             if (ramp) rc = ramp_cell(sc, c, kk / sc.n_t);
