@@ -1113,6 +1113,9 @@ static int setup_truth_bins(ms_model *m, const double *r, double rmax)
         b.nby2 = dims[k][3];
         b.r_split = k == 0 ? (float)(best_q * rmax) : 0.0f;
         b.r_max = (float)rmax;
+        // the widest skin: a radius of the first grid's floes, or in sparse ice half the
+        // mean spacing, so that a list stays a few neighbours long at any speed
+        b.skin_max = (float)std::max(best_q * rmax, 0.5 * std::sqrt(m->g.Lx * m->g.Ly / (double)std::max(n, 1LL)));
         const int nbins = b.nbins();
         b.nscan_blocks = (nbins + 1023) / 1024;
         if (b.nscan_blocks > 1024) return fail(MS_ERR_ARG, "too many bins (%d)", nbins);

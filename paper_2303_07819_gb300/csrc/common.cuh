@@ -479,6 +479,7 @@ struct TruthBins {
     int nbx, nby;          // bins per side (1 x 1: brute force)
     int nbx2, nby2;        // the large floes' grid
     float r_split, r_max;
+    float skin_max;        // truth steps: widest skin of a candidate list (m)
     __host__ __device__ int nbins() const { return nbx * nby + nbx2 * nby2; }
     int *count;            // [nbins]
     int *start;            // [nbins + 1]

@@ -20,8 +20,10 @@
 // Measured (65,341 power-law floes, FP32): 87 us a step as nine launches, 8.1 us
 // here in long runs, 78 for a call of one step with its build; 115,200 floes of
 // one size: 9.6 in long runs.
+#include <cfloat>
 #include <climits>
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "common.cuh"
 #include "truth_step.cuh"
@@ -85,6 +87,16 @@ __device__ __forceinline__ uint2 fixed(const A64 &a, const Geom &g)
     return make_uint2(fixed1(a.x, g.Lx), fixed1(a.y, g.Ly));
 }
 
+// Is the floe anywhere in the domain?  An FP64 position is not once it is NaN,
+// or so far off (above 1e15 domains in a step) that its remainder has no
+// digit left: all such floes would lie in the bins at the domain's edge, each
+// a candidate of all others.  A fixed-point position always is.
+__device__ __forceinline__ bool placed(const A32 &, const Geom &) { return true; }
+__device__ __forceinline__ bool placed(const A64 &a, const Geom &g)
+{
+    return a.x >= 0.0 && a.x <= g.Lx && a.y >= 0.0 && a.y <= g.Ly;
+}
+
 // fixed-point separation in metres: the periodic minimum image, or between
 // walls the plain difference
 __device__ __forceinline__ float sep_x(uint32_t a, uint32_t b, float sx, bool walls)
@@ -101,7 +113,7 @@ template <class F>
 __device__ __forceinline__ void visit_ranges(const int *start, int base, int nbx, int nby, uint2 q, float rx, float ry,
                                              bool walls, F &&f)
 {
-    // margin against rounding; NaN (a diverged state) takes every bin
+    // margin against rounding
     const int kx = rx * 1.0001f < (float)nbx ? (int)ceilf(rx * 1.0001f) : nbx;
     const int ky = ry * 1.0001f < (float)nby ? (int)ceilf(ry * 1.0001f) : nby;
     const int bx = fbin(q.x, nbx), by = fbin(q.y, nby);
@@ -326,6 +338,9 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
     unsigned long long ndeep = 0;
     bool bad = false;
 
+    // a floe's speed as the skins count it: at most what fills the widest skin
+    // (NaN too)
+    auto speed_of = [&](float u, float v) { return fminf(sqrtf(u * u + v * v), tb.skin_max / (48.0f * (float)a.dt)); };
     // a sum of the floes' speeds over the grid into ctl[at]; the order of its
     // additions varies, and with it the skins, but no result
     auto add_speeds = [&](float vs, int at) {
@@ -342,7 +357,7 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
     for (long long l = gt; l < n; l += gs) {
         w.A[0][l] = load_a(in, l);
         w.B[0][l] = {in.u[l], in.v[l], in.w[l], in.th[l]};
-        vs0 += hypotf((float)in.u[l], (float)in.v[l]);
+        vs0 += speed_of((float)in.u[l], (float)in.v[l]);
     }
     for (long long i = gt; i < nbins; i += gs) tb.count[i] = 0;
     for (long long i = gt; i < nsteps; i += gs) {
@@ -362,17 +377,18 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
         if (gt == 0) w.ctl[(s + 1) % 3] = 0;      // read at the last step, written at the next
         if (need) {
             // count the floes of each bin; skins: 48 steps' way at the current speed,
-            // or at half the mean one (at the build before), plus 2 % of the radius
+            // or at half the mean one (at the build before), plus 2 % of the radius,
+            // none wider than skin_max: a fast floe leaves its skin sooner, and a state
+            // that diverges keeps lists of bounded length
             float smax = 0.0f, vsum = 0.0f;
             const float vfloor = 0.5f * __int_as_float(*(volatile int *)&w.ctl[5 + (par ^ 1)]) / (float)n;
             for (long long l = gt; l < n; l += gs) {
                 const A p = w.A[cur][l];
                 const Rest<R> q = w.B[cur][l];
                 const uint2 x = fixed(p, a.g);
-                const float u = (float)q.u, v = (float)q.v, r = (float)p.r;
-                const float speed = sqrtf(u * u + v * v);
+                const float r = (float)p.r, speed = speed_of((float)q.u, (float)q.v);
                 vsum += speed;
-                const float skin = 48.0f * (float)a.dt * fmaxf(speed, vfloor) + 0.02f * r;
+                const float skin = fminf(48.0f * (float)a.dt * fmaxf(speed, vfloor), tb.skin_max) + 0.02f * r;
                 w.skin[l] = skin;
                 w.xb[l] = x;
                 smax = fmaxf(smax, skin);
@@ -416,7 +432,9 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
             for (long long l = gt; l < n; l += gs) {
                 const uint2 x = w.xb[l];
                 // the reach covers the rounding of the FP32 tests
-                const float reach = ((float)w.A[cur][l].r + w.skin[l]) * 1.00001f + 1.0e-9f * fmaxf(Lx, Ly);
+                // (negative: a floe that is nowhere touches none)
+                const A p = w.A[cur][l];
+                const float reach = placed(p, a.g) ? ((float)p.r + w.skin[l]) * 1.00001f + 1.0e-9f * fmaxf(Lx, Ly) : -FLT_MAX;
                 w.sorted[tb.start[w.binof[l]] + w.rank[l]] = {x.x, x.y, reach, (int)l};
             }
             grid.sync();
@@ -426,12 +444,13 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
         const float smax = __int_as_float(*(volatile int *)&w.ctl[3 + (par ^ 1)]);
         // f(floe, fixed-point x, y, reach) over the floes that floe l at build
         // position x with its own reach may touch
+        constexpr bool unplaced = std::is_same<A, A64>::value;   // may a reach be negative?
         auto near = [&](uint2 x, float own, auto &&f) {
             auto range = [&](int i0, int i1) {
                 for (int i = i0; i < i1; i++) {
                     const Sorted q = w.sorted[i];
                     const float dx = sep_x(q.x, x.x, sx, walls), dy = (float)(int)(q.y - x.y) * sy, r = own + q.reach;
-                    if (!(dx * dx + dy * dy >= r * r)) f(q.l);   // NaN passes
+                    if (!(dx * dx + dy * dy >= r * (unplaced ? fabsf(r) : r))) f(q.l);
                 }
             };
             const float r1 = own + (tb.r_split + smax) * 1.00001f, r2 = own + (tb.r_max + smax) * 1.00001f;
@@ -443,11 +462,13 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
         if (need) {
             for (long long l = gt; l < n; l += gs) {
                 int c = 0;
-                near(w.xb[l], own_reach(l, w.A[cur][l].r), [&](int j) {
-                    if (j == (int)l) return;
-                    if (c < LT) w.list[c * n + l] = j;
-                    c++;
-                });
+                const A p = w.A[cur][l];
+                if (placed(p, a.g))
+                    near(w.xb[l], own_reach(l, p.r), [&](int j) {
+                        if (j == (int)l) return;
+                        if (c < LT) w.list[c * n + l] = j;
+                        c++;
+                    });
                 w.cnt[l] = c;
                 if (c > 1 && c <= 16) sort_list<16>(w.list + l, n, c);
                 else if (c > 16 && c <= LT) sort_list<LT>(w.list + l, n, c);

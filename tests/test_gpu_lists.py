@@ -3,6 +3,8 @@ truth DEM where their upkeep is at its limits: rebuilt at every step, longer
 than their room, of floes far from the mean speed, radius or density.
 Tolerances as in the parity tests: 1e-10 (FP64) and 1e-4 (FP32), relative,
 per moment column."""
+import time
+
 import numpy as np
 import pytest
 
@@ -46,3 +48,61 @@ def test_fp64_lists_made_at_every_step(orc, ms, n, threads):
     e = rel_errors(a.moments(), o.moments(), p, TOL[1][1])
     assert e.max() <= TOL[1][0], report(e)
     assert same_floes(a.floes(), b.floes())
+
+
+def packed(n, L, seed=5):
+    """n floes of about 0.3 spacings on a jittered lattice over an L x L domain, at rest."""
+    rng = np.random.default_rng(seed)
+    k = int(np.ceil(np.sqrt(n)))
+    d = L / k
+    i = np.arange(n)
+    f = {key: np.zeros(n) for key in ("x", "y", "theta", "u", "v", "omega", "r", "h")}
+    f["x"] = (i % k + 0.5 + rng.uniform(-0.2, 0.2, n)) * d
+    f["y"] = (i // k + 0.5 + rng.uniform(-0.2, 0.2, n)) * d
+    f["r"] = rng.uniform(0.25, 0.35, n) * d
+    f["h"] = rng.uniform(0.5, 2.0, n)
+    return f
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", [90, 900, 3000])
+def test_truth_fast_floes(orc, ms, precision, n):
+    """All floes at tens of metres a step and one faster still: wider
+    skins than a list may have, so lists are made again every few steps.  The
+    oracle's moments, and the same floes however the run is split."""
+    L = 30e3
+    f, p = packed(n, L), dict(soft(2, L), couple=0)
+    rng = np.random.default_rng(n)
+    f["u"], f["v"] = rng.uniform(-40.0, 40.0, n), rng.uniform(-40.0, 40.0, n)
+    f["u"][n // 2] = 100.0
+    o = orc.Truth(p, f)
+    a, b = ms.Model(p, f, precision), ms.Model(p, f, precision)
+    o.step(0.5, 24)
+    a.truth_step(0.5, 24)
+    for k in (1, 7, 16):
+        b.truth_step(0.5, k)
+    e = rel_errors(a.truth_moments(), o.moments(), p, TOL[precision][1])
+    assert e.max() <= TOL[precision][0], report(e)
+    assert same_floes(a.truth_floes(), b.truth_floes())
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_truth_diverged_state(ms, precision):
+    """Every floe at 1e12 m/s: the speeds turn inf and NaN within a few steps,
+    from which no list may grow with the number of floes.  60,000 floes, 200
+    steps: with lists of a few neighbours, made at every step, some 0.1 ms a
+    step; had every floe the others as candidates, 4e9 tests a step.  The
+    step reports MS_ERR_UNSTABLE and the context stays usable."""
+    n, L = 60_000, 300e3
+    f, p = packed(n, L), dict(soft(8, L), couple=0)
+    f["u"][:] = 1.0e12
+    m = ms.Model(p, f, precision)
+    t = time.perf_counter()
+    with pytest.raises(ms.MsError) as e:
+        m.truth_step(10.0, 200)
+    assert e.value.code == -3, str(e.value)
+    assert time.perf_counter() - t < 1.0
+    f["u"][:] = 0.0
+    m = ms.Model(p, f, precision)
+    m.truth_step(10.0, 3)
+    assert np.all(np.isfinite(m.truth_moments()))
