@@ -35,7 +35,8 @@ namespace msd {
 namespace {
 
 constexpr int TT = 256;       // threads per block
-constexpr int LT = 64;        // candidates per floe; a floe with more searches its bins at every step
+constexpr int LT = 64;        // candidates per floe; the warp searches the bins of a floe with more at every step
+constexpr int FOUND = 256;    // touching partners such a search holds
 
 // a floe in the working copy: what a contact test reads, and the rest
 struct A32 { uint32_t x, y; float r, h; };
@@ -108,9 +109,10 @@ __device__ __forceinline__ int fbin(uint32_t q, int nb) { return (int)(((unsigne
 
 // Calls f(first, last + 1) for the ranges of sorted floes in the bins of one
 // grid (nbx x nby bins from bin `base`) within (rx, ry) bin sides of the bin
-// that holds a floe at fixed point q; bins side by side in x are one range.
+// that holds a floe at fixed point q, until f returns false (then so does this); bins side by
+// side in x are one range.
 template <class F>
-__device__ __forceinline__ void visit_ranges(const int *start, int base, int nbx, int nby, uint2 q, float rx, float ry,
+__device__ __forceinline__ bool visit_ranges(const int *start, int base, int nbx, int nby, uint2 q, float rx, float ry,
                                              bool walls, F &&f)
 {
     // margin against rounding
@@ -124,16 +126,17 @@ __device__ __forceinline__ void visit_ranges(const int *start, int base, int nbx
         cy = cy < 0 ? cy + nby : (cy >= nby ? cy - nby : cy);
         const int *row = start + base + cy * nbx;
         if (allx) {
-            f(row[0], row[nbx]);
+            if (!f(row[0], row[nbx])) return false;
             continue;
         }
         const int lo = bx - kx, hi = bx + kx;
-        f(row[max(lo, 0)], row[min(hi, nbx - 1) + 1]);
+        if (!f(row[max(lo, 0)], row[min(hi, nbx - 1) + 1])) return false;
         if (!walls) {
-            if (lo < 0) f(row[lo + nbx], row[nbx]);
-            if (hi >= nbx) f(row[0], row[hi - nbx + 1]);
+            if (lo < 0 && !f(row[lo + nbx], row[nbx])) return false;
+            if (hi >= nbx && !f(row[0], row[hi - nbx + 1])) return false;
         }
     }
+    return true;
 }
 
 // ascending sort of v[0..N) in registers (bitonic, every index static)
@@ -297,6 +300,146 @@ __device__ __forceinline__ A64 moved(const A64 &a, const TruthArgs &t, bool wall
     return b;
 }
 
+// A floe's reach: its radius, its skin and what covers the rounding of the
+// FP32 tests (negative: a floe that is nowhere touches none).
+template <class A>
+__device__ __forceinline__ float reach_of(const A &p, float skin, const Geom &g)
+{
+    return placed(p, g) ? ((float)p.r + skin) * 1.00001f + 1.0e-9f * fmaxf((float)g.Lx, (float)g.Ly) : -FLT_MAX;
+}
+
+// Calls f(first, last + 1) for the ranges of w.sorted that hold every floe
+// within reach of one at build position x with reach `own`, until f returns
+// false; smax: the largest skin.
+template <class T, class F>
+__device__ __forceinline__ void near_ranges(const Work<T> &w, const TruthArgs &a, const TruthBins &tb, uint2 x, float own,
+                                            float smax, F &&f)
+{
+    const bool walls = a.g.walls != 0;
+    const float Lx = (float)a.g.Lx, Ly = (float)a.g.Ly;
+    const float r1 = own + (tb.r_split + smax) * 1.00001f, r2 = own + (tb.r_max + smax) * 1.00001f;
+    if (visit_ranges(tb.start, 0, tb.nbx, tb.nby, x, r1 * tb.nbx / Lx, r1 * tb.nby / Ly, walls, f) && tb.nbx2 > 0)
+        visit_ranges(tb.start, tb.nbx * tb.nby, tb.nbx2, tb.nby2, x, r2 * tb.nbx2 / Lx, r2 * tb.nby2 / Ly, walls, f);
+}
+
+// were the two floes within reach at the build?
+template <class T>
+__device__ __forceinline__ bool in_reach(const Sorted &q, uint2 x, float own, const TruthArgs &a)
+{
+    constexpr bool unplaced = std::is_same<T, Tr64>::value;      // may a reach be negative?
+    const float dx = sep_x(q.x, x.x, a.k.sx, a.g.walls != 0), dy = (float)(int)(q.y - x.y) * a.k.sy, r = own + q.reach;
+    return !(dx * dx + dy * dy >= r * (unplaced ? fabsf(r) : r));
+}
+
+// the warp's numbers v[0..m), all different, into ascending order (m <= FOUND)
+__device__ __forceinline__ void sort_warp(int *v, int m)
+{
+    const int lane = threadIdx.x & 31;
+    int x[FOUND / 32], rank[FOUND / 32];
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < FOUND / 32; k++) {
+        x[k] = lane + 32 * k < m ? v[lane + 32 * k] : 0;
+        rank[k] = 0;
+    }
+    for (int i = 0; i < m; i++) {
+        const int o = v[i];
+#pragma unroll
+        for (int k = 0; k < FOUND / 32; k++) rank[k] += o < x[k] ? 1 : 0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < FOUND / 32; k++)
+        if (lane + 32 * k < m) v[rank[k]] = x[k];
+    __syncwarp();
+}
+
+// Floes with more candidates than a list holds, of one warp's 32: their
+// contacts are found by the whole warp, a candidate a lane, and handed to the
+// floe's lane in portions of up to LT, in ascending order.  (One lane
+// searching for one contact after another took 0.3 ms a step for a floe of
+// 19 km among floes of 0.2 km, the search of all bins once a step before 0.19.)
+struct LongLists {
+    unsigned left;         // lanes whose floes are still to be searched
+    int src, at, held;     // the floe's lane; the next partner to hand on, partners found
+    int above;             // its partners up to this one are done with
+    int more;              // are there more than were held?
+    int found[FOUND];
+};
+
+// The next portion into the list of its floe: to the floe's lane the number of
+// partners, 0 to the others, -1 to all if there is none left.  l0: the floe
+// of lane 0.  (Not inlined: its registers are its own.)
+template <class T>
+__device__ __noinline__ int next_portion(const Work<T> &w, const TruthArgs &a, const TruthBins &tb,
+                                         const typename T::A *A, long long l0, float smax, LongLists &S)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    unsigned left = S.left;
+    int src = S.src, at = S.at, held = S.held, above = S.above, more = S.more;
+    __syncwarp();
+    while (at == held) {
+        if (!more) {
+            if (left == 0u) return -1;
+            src = __ffs((int)left) - 1;
+            left &= left - 1u;
+            above = -1;
+        }
+        const int l = (int)l0 + src;
+        const typename T::A me = A[l];
+        const uint2 x = w.xb[l];
+        const float own = reach_of(me, w.skin[l], a.g);
+        const bool walls = a.g.walls != 0;
+        int m = 0, lim = INT_MAX;
+        near_ranges<T>(w, a, tb, x, own, smax, [&](int i0, int i1) {
+            for (; i0 < i1; i0 += 32) {
+                bool hit = false;
+                int j = 0;
+                if (i0 + lane < i1) {
+                    const Sorted q = w.sorted[i0 + lane];
+                    j = q.l;
+                    if (j != l && j > above && j < lim && in_reach<T>(q, x, own, a)) {
+                        typename T::R dx, dy;
+                        const typename T::A o = A[j];
+                        pair_xy(o, me, a, walls, dx, dy);
+                        const typename T::R r = me.r + o.r;
+                        hit = dx * dx + dy * dy < r * r * typename T::R(1.00001);   // the walk decides
+                    }
+                }
+                const unsigned hits = __ballot_sync(FULL, hit);
+                if (hit) S.found[m + __popc(hits & ((1u << lane) - 1u))] = j;
+                m += __popc(hits);
+                if (m > FOUND - 32) {      // the smaller half, and from here on only what belongs among it
+                    sort_warp(S.found, m);
+                    m = FOUND / 2;
+                    lim = S.found[m];
+                    __syncwarp();          // (read by all before the next is put there)
+                }
+            }
+            return true;
+        });
+        sort_warp(S.found, m);
+        more = lim != INT_MAX;
+        at = 0;
+        held = m;
+        if (more) above = lim - 1;
+    }
+    const int k = min(LT, held - at);
+    for (int i = lane; i < k; i += 32) w.list[i * a.n + l0 + src] = S.found[at + i];
+    if (lane == 0) {
+        S.left = left;
+        S.src = src;
+        S.at = at + k;
+        S.held = held;
+        S.above = above;
+        S.more = more;
+    }
+    __syncwarp();
+    return lane == src ? k : 0;
+}
+
 // exclusive scan of one value per thread over the block; total to all threads
 __device__ __forceinline__ int block_excl(int v, int *ws, int &total)
 {
@@ -322,18 +465,19 @@ __device__ __forceinline__ int block_excl(int v, int *ws, int &total)
 
 template <class T>
 __global__ void __launch_bounds__(TT)
-k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, TruthArgs a, TruthBins tb, Work<T> w,
-            int nsteps)
+k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, const __grid_constant__ TruthArgs a,
+            const __grid_constant__ TruthBins tb, const __grid_constant__ Work<T> w, int nsteps)
 {
     using R = typename T::R;
     using A = typename T::A;
     cg::grid_group grid = cg::this_grid();
     __shared__ int ws[TT / 32];
     __shared__ float wmax[TT / 32], wsum[TT / 32];
+    __shared__ LongLists longs[TT / 32];
     const long long n = a.n, gt = blockIdx.x * (long long)TT + threadIdx.x, gs = gridDim.x * (long long)TT;
     const bool walls = a.g.walls != 0;
     const int nbins = tb.nbins(), nb1 = tb.nbx * tb.nby;
-    const float sx = a.k.sx, sy = a.k.sy, Lx = (float)a.g.Lx, Ly = (float)a.g.Ly;
+    const float sx = a.k.sx, sy = a.k.sy;
     R *fd = reinterpret_cast<R *>(a.fd);
     unsigned long long ndeep = 0;
     bool bad = false;
@@ -431,10 +575,7 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
             grid.sync();
             for (long long l = gt; l < n; l += gs) {
                 const uint2 x = w.xb[l];
-                // the reach covers the rounding of the FP32 tests
-                // (negative: a floe that is nowhere touches none)
-                const A p = w.A[cur][l];
-                const float reach = placed(p, a.g) ? ((float)p.r + w.skin[l]) * 1.00001f + 1.0e-9f * fmaxf(Lx, Ly) : -FLT_MAX;
+                const float reach = reach_of(w.A[cur][l], w.skin[l], a.g);
                 w.sorted[tb.start[w.binof[l]] + w.rank[l]] = {x.x, x.y, reach, (int)l};
             }
             grid.sync();
@@ -442,32 +583,21 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
         // the largest skin of the lists in use (of either parity's build)
         if (need) par ^= 1;
         const float smax = __int_as_float(*(volatile int *)&w.ctl[3 + (par ^ 1)]);
-        // f(floe, fixed-point x, y, reach) over the floes that floe l at build
-        // position x with its own reach may touch
-        constexpr bool unplaced = std::is_same<A, A64>::value;   // may a reach be negative?
-        auto near = [&](uint2 x, float own, auto &&f) {
-            auto range = [&](int i0, int i1) {
-                for (int i = i0; i < i1; i++) {
-                    const Sorted q = w.sorted[i];
-                    const float dx = sep_x(q.x, x.x, sx, walls), dy = (float)(int)(q.y - x.y) * sy, r = own + q.reach;
-                    if (!(dx * dx + dy * dy >= r * (unplaced ? fabsf(r) : r))) f(q.l);
-                }
-            };
-            const float r1 = own + (tb.r_split + smax) * 1.00001f, r2 = own + (tb.r_max + smax) * 1.00001f;
-            visit_ranges(tb.start, 0, tb.nbx, tb.nby, x, r1 * tb.nbx / Lx, r1 * tb.nby / Ly, walls, range);
-            if (tb.nbx2 > 0)
-                visit_ranges(tb.start, nb1, tb.nbx2, tb.nby2, x, r2 * tb.nbx2 / Lx, r2 * tb.nby2 / Ly, walls, range);
-        };
-        auto own_reach = [&](long long l, R r) { return ((float)r + w.skin[l]) * 1.00001f + 1.0e-9f * fmaxf(Lx, Ly); };
         if (need) {
             for (long long l = gt; l < n; l += gs) {
                 int c = 0;
                 const A p = w.A[cur][l];
+                const uint2 x = w.xb[l];
+                const float own = reach_of(p, w.skin[l], a.g);
                 if (placed(p, a.g))
-                    near(w.xb[l], own_reach(l, p.r), [&](int j) {
-                        if (j == (int)l) return;
-                        if (c < LT) w.list[c * n + l] = j;
-                        c++;
+                    near_ranges<T>(w, a, tb, x, own, smax, [&](int i0, int i1) {
+                        for (int i = i0; i < i1 && c <= LT; i++) {   // (one more than a list holds is all there is to know)
+                            const Sorted q = w.sorted[i];
+                            if (q.l == (int)l || !in_reach<T>(q, x, own, a)) continue;
+                            if (c < LT) w.list[c * n + l] = q.l;
+                            c++;
+                        }
+                        return c <= LT;
                     });
                 w.cnt[l] = c;
                 if (c > 1 && c <= 16) sort_list<16>(w.list + l, n, c);
@@ -477,22 +607,27 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
         const bool last = s == nsteps - 1;
         const double2 wa = w.wind[s];
         bool far = false;
-        for (long long l = gt; l < n; l += gs) {
+        for (long long l0 = gt - (threadIdx.x & 31); l0 < n; l0 += gs) {      // a warp's 32 floes
+            const bool valid = l0 + (threadIdx.x & 31) < n;
+            const long long l = valid ? l0 + (threadIdx.x & 31) : l0;
             const A me = w.A[cur][l];
             const Rest<R> q = w.B[cur][l];
             R fx = 0, fy = 0, tq = 0;
             unsigned deep = 0;
-            auto contact = [&](int j, const A &o) {
-                R dx, dy;
-                pair_xy(o, me, a, walls, dx, dy);
-                const R d2 = dx * dx + dy * dy, S = me.r + o.r;
-                if (d2 < S * S) {
-                    const Rest<R> p = w.B[cur][j];
-                    contact_add(dx, dy, d2, me.r, o.r, me.h, o.h, p.u - q.u, p.v - q.v, q.w, p.w, P, fx, fy, tq, deep);
+            int c = valid ? w.cnt[l] : 0;
+            const bool any_long = __any_sync(0xffffffffu, c > LT);
+            if (any_long) {
+                const unsigned left = __ballot_sync(0xffffffffu, c > LT);
+                if ((threadIdx.x & 31) == 0) {
+                    LongLists &S = longs[threadIdx.x >> 5];
+                    S.left = left;
+                    S.at = S.held = S.more = 0;
                 }
-            };
-            const int c = w.cnt[l];
-            if (c <= LT) {
+                if (c > LT) c = 0;
+            }
+            // the floe's list, contacts in ascending partner order (the portions of a
+            // long one take the same way, so its forces are rounded alike)
+            do {
                 for (int i = 0; i < c; i += 4) {      // four partners' loads in flight
                     int j[4];
                     A o[4];
@@ -501,29 +636,21 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
 #pragma unroll
                     for (int k = 0; k < 4; k++) o[k] = w.A[cur][j[k]];
 #pragma unroll
-                    for (int k = 0; k < 4; k++)
-                        if (i + k < c) contact(j[k], o[k]);
-                }
-            } else {
-                // more candidates than a list holds: the smallest partner above the
-                // last one, until there is none
-                const uint2 x = w.xb[l];
-                const float own = own_reach(l, me.r);
-                for (int lastj = -1;;) {
-                    int best = INT_MAX;
-                    near(x, own, [&](int j) {
-                        if (j <= lastj || j >= best || j == (int)l) return;
+                    for (int k = 0; k < 4; k++) {
+                        if (i + k >= c) continue;
                         R dx, dy;
-                        const A o = w.A[cur][j];
-                        pair_xy(o, me, a, walls, dx, dy);
-                        const R S = me.r + o.r;
-                        if (dx * dx + dy * dy < S * S) best = j;
-                    });
-                    if (best == INT_MAX) break;
-                    contact(best, w.A[cur][best]);
-                    lastj = best;
+                        pair_xy(o[k], me, a, walls, dx, dy);
+                        const R d2 = dx * dx + dy * dy, S = me.r + o[k].r;
+                        if (d2 < S * S) {
+                            const Rest<R> p = w.B[cur][j[k]];
+                            contact_add(dx, dy, d2, me.r, o[k].r, me.h, o[k].h, p.u - q.u, p.v - q.v, q.w, p.w, P, fx, fy,
+                                        tq, deep);
+                        }
+                    }
                 }
-            }
+                if (any_long) c = next_portion<T>(w, a, tb, w.A[cur], l0, smax, longs[threadIdx.x >> 5]);
+            } while (any_long && c >= 0);
+            if (!valid) continue;
             R uo, vo, zeta;
             ocean_at(P, w, a, me, uo, vo, zeta);
             if (walls) wall_force(me, a, q.u, q.v, q.w, P, fx, fy, tq, deep);

@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 from tests.parity import rel_errors, report
-from tests.test_gpu_runs import TOL, crowd, join, soft
+from tests.test_gpu_runs import TOL, crowd, join, ring, soft
 
 pytestmark = pytest.mark.gpu
 
@@ -106,3 +106,44 @@ def test_truth_diverged_state(ms, precision):
     m = ms.Model(p, f, precision)
     m.truth_step(10.0, 3)
     assert np.all(np.isfinite(m.truth_moments()))
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n,small", [(63, 300.0), (64, 300.0), (65, 250.0), (130, 200.0), (220, 80.0), (230, 80.0), (900, 20.0)])
+def test_truth_long_lists(orc, ms, precision, n, small):
+    """Two large floes of one warp, one of them across the domain's corner,
+    each with up to n partners: lists of just up to 64, portions of 64 of longer
+    ones, and more partners than one search of the warp holds.  The oracle's
+    moments, and the same floes however the run is split."""
+    L = 100e3
+    parts = [ring(n, L, 6000.0, small), ring(n, L, 5900.0, small)]
+    parts[0]["x"] = np.mod(parts[0]["x"] + 0.5 * L, L)
+    parts[0]["y"] = np.mod(parts[0]["y"] + 0.5 * L, L)
+    f = join(parts)
+    order = np.r_[0, n + 1, 1:n + 1, n + 2:2 * n + 2]
+    f, p = {k: v[order] for k, v in f.items()}, dict(soft(4, L), couple=0)
+    o = orc.Truth(p, f)
+    a, b = ms.Model(p, f, precision), ms.Model(p, f, precision)
+    o.step(10.0, 23)
+    a.truth_step(10.0, 23)
+    for k in (1, 7, 15):
+        b.truth_step(10.0, k)
+    e = rel_errors(a.truth_moments(), o.moments(), p, TOL[precision][1])
+    assert e.max() <= TOL[precision][0], report(e)
+    assert same_floes(a.truth_floes(), b.truth_floes())
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_truth_diverged_between_walls(ms, precision):
+    """As test_truth_diverged_state, between walls: within two steps all
+    floes stand on a wall, some 140 to a bin's side, each with as many
+    partners.  20,000 floes, 200 steps: a few ms a step at most."""
+    n, L = 20_000, 170e3
+    f, p = packed(n, L), dict(soft(8, L), couple=0, walls=1)
+    f["u"][:] = 1.0e12
+    m = ms.Model(p, f, precision)
+    t = time.perf_counter()
+    with pytest.raises(ms.MsError) as e:
+        m.truth_step(10.0, 200)
+    assert e.value.code == -3, str(e.value)
+    assert time.perf_counter() - t < 1.0
