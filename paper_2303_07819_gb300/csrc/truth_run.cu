@@ -20,6 +20,7 @@
 // Measured (65,341 power-law floes, FP32): 87 us a step as nine launches, 8.1 us
 // here in long runs, 78 for a call of one step with its build; 115,200 floes of
 // one size: 9.6 in long runs.
+#include <algorithm>
 #include <cfloat>
 #include <climits>
 #include <cooperative_groups.h>
@@ -520,11 +521,14 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
         const bool need = *(volatile int *)&w.ctl[(s + 2) % 3] != 0;
         if (gt == 0) w.ctl[(s + 1) % 3] = 0;      // read at the last step, written at the next
         if (need) {
-            // count the floes of each bin; skins: 48 steps' way at the current speed,
-            // or at half the mean one (at the build before), plus 2 % of the radius,
-            // none wider than skin_max: a fast floe leaves its skin sooner, and a state
-            // that diverges keeps lists of bounded length
+            // count the floes of each bin; skins: 48 steps' way (in a launch's last
+            // twelve, four times what is left: a call of one step needs no longer
+            // lists) at the current speed, or at half the mean one (at the build
+            // before), plus 2 % of the radius, none wider than skin_max: a fast floe
+            // leaves its skin sooner, and a state that diverges keeps lists of
+            // bounded length
             float smax = 0.0f, vsum = 0.0f;
+            const float ahead = (float)a.dt * (float)min(48, 4 * (nsteps - s));
             const float vfloor = 0.5f * __int_as_float(*(volatile int *)&w.ctl[5 + (par ^ 1)]) / (float)n;
             for (long long l = gt; l < n; l += gs) {
                 const A p = w.A[cur][l];
@@ -532,7 +536,7 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
                 const uint2 x = fixed(p, a.g);
                 const float r = (float)p.r, speed = speed_of((float)q.u, (float)q.v);
                 vsum += speed;
-                const float skin = fminf(48.0f * (float)a.dt * fmaxf(speed, vfloor), tb.skin_max) + 0.02f * r;
+                const float skin = fminf(ahead * fmaxf(speed, vfloor), tb.skin_max) + 0.02f * r;
                 w.skin[l] = skin;
                 w.xb[l] = x;
                 smax = fmaxf(smax, skin);
@@ -551,13 +555,13 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
             }
             add_speeds(vsum, 5 + par);
             grid.sync();
-            // each block a run of bins: its total, then the starts
-            const int per = (nbins + gridDim.x - 1) / gridDim.x;
-            const int c0 = min((int)blockIdx.x * per, nbins), c1 = min(c0 + per, nbins);
-            const int each = (per + TT - 1) / TT;
-            const int t0 = min(c0 + (int)threadIdx.x * each, c1), t1 = min(t0 + each, c1);
+            // each warp a run of bins, a bin a lane: the blocks' totals, then the
+            // starts
+            const int per = ((nbins + (int)gridDim.x * (TT / 32) - 1) / ((int)gridDim.x * (TT / 32)) + 31) & ~31;
+            const int c0 = (int)min((long long)(blockIdx.x * (TT / 32) + (threadIdx.x >> 5)) * per, (long long)nbins);
+            const int c1 = min(c0 + per, nbins), lane = threadIdx.x & 31;
             int sum = 0;
-            for (int i = t0; i < t1; i++) sum += tb.count[i];
+            for (int i = c0 + lane; i < c1; i += 32) sum += tb.count[i];
             int total;
             const int mine = block_excl(sum, ws, total);
             if (threadIdx.x == 0) w.bsum[blockIdx.x] = total;
@@ -566,11 +570,20 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
             int before = 0;
             for (int i = threadIdx.x; i < (int)blockIdx.x; i += TT) before += w.bsum[i];
             block_excl(before, ws, before);
-            int run = before + mine;
-            for (int i = t0; i < t1; i++) {
-                tb.start[i] = run;
-                run += tb.count[i];
-                tb.count[i] = 0;
+            int run = before + __shfl_sync(0xffffffffu, mine, 0);
+            for (int i0 = c0; i0 < c1; i0 += 32) {
+                const int c = i0 + lane < c1 ? tb.count[i0 + lane] : 0;
+                int x = c;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, x, d);
+                    if (lane >= d) x += y;
+                }
+                if (i0 + lane < c1) {
+                    tb.start[i0 + lane] = run + x - c;
+                    tb.count[i0 + lane] = 0;
+                }
+                run += __shfl_sync(0xffffffffu, x, 31);
             }
             grid.sync();
             for (long long l = gt; l < n; l += gs) {
@@ -690,8 +703,12 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
     if (ndeep) atomicAdd(&a.ctrl->deep, ndeep);
 }
 
+// Blocks for n floes or, in sparse ice, for a bin of every 32 to a thread: a
+// build goes over all bins (500 floes of 50 m in 100 km, a million bins, a call
+// of one step: 2650 us on the two blocks of their floes, 52 so; blocks for a
+// bin of every 8 to a thread: 52, but 4.5 us a step in long runs instead of 4.1).
 template <class T>
-int grid_of(long long n)
+int grid_of(long long n, int nbins)
 {
     static int per_sm = 0, nsm = 0;
     if (!per_sm) {
@@ -701,7 +718,7 @@ int grid_of(long long n)
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_truth_run<T>, TT, 0) != cudaSuccess) b = 0;
         per_sm = b > 0 ? b : 1;
     }
-    const long long need = (n + TT - 1) / TT, most = (long long)per_sm * nsm;
+    const long long need = (std::max<long long>(n, nbins / 32) + TT - 1) / TT, most = (long long)per_sm * nsm;
     return (int)(need < 1 ? 1 : (need < most ? need : most));
 }
 
@@ -748,7 +765,8 @@ cudaError_t launch(const typename T::State &in, const typename T::State &out, co
     Phys<typename T::R> p = P;
     TruthArgs ta = a;
     void *args[] = {&si, &so, &p, &ta, &b, &w, &nsteps};
-    return cudaLaunchCooperativeKernel((const void *)k_truth_run<T>, dim3(grid_of<T>(a.n)), dim3(TT), args, 0, st);
+    return cudaLaunchCooperativeKernel((const void *)k_truth_run<T>, dim3(grid_of<T>(a.n, b.nbins())), dim3(TT), args, 0,
+                                       st);
 }
 
 }  // namespace

@@ -147,3 +147,29 @@ def test_truth_diverged_between_walls(ms, precision):
         m.truth_step(10.0, 200)
     assert e.value.code == -3, str(e.value)
     assert time.perf_counter() - t < 1.0
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n,r", [(2, 40.0), (500, 50.0), (1500, 60.0), (333, 777.0)])
+def test_truth_sparse(orc, ms, precision, n, r):
+    """Touching pairs far from each other, up to a million bins to a few
+    floes: the oracle's moments, the same floes however the run is split, and
+    no call of one step that goes over all bins on the few blocks of the
+    floes (which took 2.6 ms; a call costs some 0.05)."""
+    L = 100e3
+    f, p = packed(n, L), dict(soft(4, L), couple=0)
+    f["r"][:] = r
+    f["x"][1::2], f["y"][1::2] = np.mod(f["x"][:n - n % 2:2] + 1.9 * r, L), f["y"][:n - n % 2:2]
+    o = orc.Truth(p, f)
+    a, b = ms.Model(p, f, precision), ms.Model(p, f, precision)
+    o.step(10.0, 23)
+    a.truth_step(10.0, 23)
+    t = []
+    for _ in range(23):
+        t0 = time.perf_counter()
+        b.truth_step(10.0, 1)
+        t.append(time.perf_counter() - t0)
+    e = rel_errors(a.truth_moments(), o.moments(), p, TOL[precision][1])
+    assert e.max() <= TOL[precision][0], report(e)
+    assert same_floes(a.truth_floes(), b.truth_floes())
+    assert np.median(t) < 1.0e-3
