@@ -1247,20 +1247,26 @@ cudaError_t run_block_prepare()
 // (at most one per group).
 static int run_block_grid(int K, int ngroups)
 {
-    static int blocks_per_sm[3] = {0, 0, 0}, nsm = 0;
-    const int ki = K == 1 ? 0 : (K == 2 ? 1 : 2);
-    if (!blocks_per_sm[ki]) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        const int b = with_class(K, [](auto kern, int threads, size_t sm) {
-            int n = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, sm);
-            return n;
-        });
-        blocks_per_sm[ki] = b > 0 ? b : 1;
-    }
-    const int g = blocks_per_sm[ki] * (nsm > 0 ? nsm : 1);
+    // (made by the first caller; others wait for it)
+    struct Most {
+        int of[3];
+        Most()
+        {
+            int dev = 0, nsm = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+            for (int i = 0; i < 3; i++) {
+                const int b = with_class(1 << i, [](auto kern, int threads, size_t sm) {
+                    int n = 0;
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, sm);
+                    return n;
+                });
+                of[i] = (b > 0 ? b : 1) * (nsm > 0 ? nsm : 1);
+            }
+        }
+    };
+    static const Most most;
+    const int g = most.of[K == 1 ? 0 : (K == 2 ? 1 : 2)];
     return g < ngroups ? g : ngroups;
 }
 

@@ -11,6 +11,7 @@
 // One block owns one cell at a time, so the update is in place: the block
 // reads its whole cell into shared memory before any thread writes.
 #include <cmath>
+#include <mutex>
 
 #include "common.cuh"
 
@@ -2343,9 +2344,11 @@ size_t cell_step_smem(int precision, const CellLaunch &cl, int max_n, int, int)
 
 cudaError_t cell_step_prepare(int, const CellLaunch &, size_t smem)
 {
-    static int done = 0;
+    static std::mutex once;               // models of several threads may come here first together
+    static bool done = false;
     static int optin = 0;
     static int limit = 0;
+    std::lock_guard<std::mutex> lock(once);
     if (!done) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
@@ -2371,7 +2374,7 @@ cudaError_t cell_step_prepare(int, const CellLaunch &, size_t smem)
             if (e != cudaSuccess) return e;
             limit = dyn < limit ? dyn : limit;
         }
-        done = 1;
+        done = true;
     }
     return smem <= (size_t)limit ? cudaSuccess : cudaErrorInvalidValue;
 }

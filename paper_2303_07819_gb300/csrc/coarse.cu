@@ -252,15 +252,15 @@ int coarse_launches() { return 1; }
 // (a cooperative launch needs them all resident), at most one per 256 cells
 static int coarse_fused_grid(int nc)
 {
-    static int per_sm = -1, nsm = 0;
-    if (per_sm < 0) {
-        int dev = 0, b = 0;
+    // (made by the first caller; others wait for it)
+    static const int most = [] {
+        int dev = 0, nsm = 0, b = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_coarse_fused, CF_T, 0) != cudaSuccess) b = 0;
-        per_sm = b;
-    }
-    const int need = (nc + CF_T - 1) / CF_T, most = per_sm * nsm;
+        return b * nsm;
+    }();
+    const int need = (nc + CF_T - 1) / CF_T;
     return need < most ? need : most;
 }
 

@@ -710,15 +710,15 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
 template <class T>
 int grid_of(long long n, int nbins)
 {
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        int dev = 0, b = 0;
+    // (made by the first caller; others wait for it)
+    static const long long most = [] {
+        int dev = 0, nsm = 0, b = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_truth_run<T>, TT, 0) != cudaSuccess) b = 0;
-        per_sm = b > 0 ? b : 1;
-    }
-    const long long need = (std::max<long long>(n, nbins / 32) + TT - 1) / TT, most = (long long)per_sm * nsm;
+        return (long long)std::max(b, 1) * nsm;
+    }();
+    const long long need = (std::max<long long>(n, nbins / 32) + TT - 1) / TT;
     return (int)(need < 1 ? 1 : (need < most ? need : most));
 }
 

@@ -3,11 +3,14 @@ truth DEM where their upkeep is at its limits: rebuilt at every step, longer
 than their room, of floes far from the mean speed, radius or density.
 Tolerances as in the parity tests: 1e-10 (FP64) and 1e-4 (FP32), relative,
 per moment column."""
+import subprocess
+import sys
 import time
 
 import numpy as np
 import pytest
 
+from tests.conftest import ROOT
 from tests.parity import rel_errors, report
 from tests.test_gpu_runs import TOL, crowd, join, ring, soft
 
@@ -173,3 +176,41 @@ def test_truth_sparse(orc, ms, precision, n, r):
     assert e.max() <= TOL[precision][0], report(e)
     assert same_floes(a.truth_floes(), b.truth_floes())
     assert np.median(t) < 1.0e-3
+
+
+def test_first_calls_of_several_threads(tmp_path):
+    """Models of several threads that make a process's first steps together
+    (launch sizes and kernel limits are worked out by whoever comes first)
+    give the floes of one model stepped alone."""
+    prog = tmp_path / "first.py"
+    prog.write_text(f"""
+import sys, threading
+sys.path.insert(0, {ROOT!r})
+import numpy as np
+from paper_2303_07819_gb300 import msdem as ms
+from tests.test_gpu_lists import packed
+from tests.test_gpu_runs import soft
+ms.load()
+out, start = [None] * 8, threading.Barrier(8)
+def one(i):
+    start.wait()
+    m = ms.Model(dict(soft(4, 100e3)), packed(900, 100e3), i % 2)
+    start.wait()
+    m.truth_step(10.0, 5)
+    m.step(10.0, 15)
+    out[i] = (m.truth_floes(), m.floes())
+th = [threading.Thread(target=one, args=(i,)) for i in range(8)]
+[t.start() for t in th]
+[t.join() for t in th]
+for p in (0, 1):
+    m = ms.Model(dict(soft(4, 100e3)), packed(900, 100e3), p)
+    m.truth_step(10.0, 5)
+    m.step(10.0, 15)
+    ref = (m.truth_floes(), m.floes())
+    for i in range(p, 8, 2):
+        for a, b in zip(out[i], ref):
+            assert all(np.array_equal(a[k], b[k]) for k in b), i
+print("same")
+""")
+    r = subprocess.run([sys.executable, str(prog)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "same" in r.stdout, r.stdout + r.stderr
