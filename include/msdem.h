@@ -16,9 +16,14 @@
  *  - Pointers marked "host" are ordinary CPU memory owned by the caller; the
  *    library copies from or into them before returning.  The library never
  *    keeps a caller pointer.
- *  - Device memory is allocated by the library (cudaMalloc) in ms_init and
- *    released by ms_free.  One model handle belongs to one host thread at a
- *    time; calls on different handles are independent.
+ *  - Device memory is allocated by the library (cudaMalloc) and released by
+ *    ms_free: in ms_init, and by the first call of a part that not every model
+ *    uses -- ms_truth_step (360 bytes a floe in FP32, 424 in FP64, and in FP64 up
+ *    to 64 MB for the current), ms_time_kernel and ms_autotune (out-of-place
+ *    state), ms_set_shard, ms_closure_attach.  A call whose
+ *    allocation fails returns MS_ERR_CUDA and may be made again.  One model
+ *    handle belongs to one host thread at a time; calls on different handles
+ *    are independent.
  *  - Every call is synchronous: when it returns, its work on the model's
  *    stream has finished and its outputs are valid.
  *  - Return value: MS_OK (0) or a negative MS_ERR_* code; ms_last_error()

@@ -18,6 +18,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "classes.cuh"
+#include "ready.h"
 #include "common.cuh"
 #include "shard.cuh"
 #include "upload.cuh"
@@ -95,7 +96,7 @@ struct ms_model {
     int tcur = 0;
     void *d_fd = nullptr;
     TruthBins tb{}, cb{};
-    unsigned char *d_twork = nullptr;   // the truth steps' work arrays (made by the first of them)
+    WorkArea twork;                     // the truth steps' work arrays (made by the first of them)
     double *d_tmom = nullptr;
     // schedule
     long long steps = 0, truth_steps = 0;
@@ -143,7 +144,10 @@ static cudaError_t dalloc(ms_model *m, T **p, size_t count)
 {
     void *q = nullptr;
     cudaError_t e = cudaMalloc(&q, sizeof(T) * (count > 0 ? count : 1));
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+        cudaGetLastError();      // not the next launch's error
+        return e;
+    }
     m->allocs.push_back(q);
     *p = reinterpret_cast<T *>(q);
     return cudaSuccess;
@@ -1792,15 +1796,14 @@ static TruthArgs truth_args(const ms_model *m, double dt, long long step)
 // nsteps <= TRUTH_CHUNK truth steps from copy cur to the other, step `step` first
 static cudaError_t truth_run(ms_model *m, int cur, long long step, int nsteps)
 {
-    if (!m->d_twork) {
-        cudaError_t e = dalloc(m, &m->d_twork, truth_work_bytes(m->precision, m->n, m->P64, m->g));
-        if (e == cudaSuccess) e = truth_work_init(m->precision, m->n, m->P64, m->g, m->d_twork, m->stream);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = make_ready(
+        m->twork, [m](unsigned char *&p) { return dalloc(m, &p, truth_work_bytes(m->precision, m->n, m->P64, m->g)); },
+        [m](unsigned char *p) { return truth_work_init(m->precision, m->n, m->P64, m->g, p, m->stream); });
+    if (e != cudaSuccess) return e;
     const TruthArgs a = truth_args(m, m->truth_dt, step);
     if (m->precision == MS_FP64)
-        return launch_truth_run64(m->t64[cur], m->t64[1 - cur], m->P64, a, m->tb, m->d_twork, nsteps, m->stream);
-    return launch_truth_run32(m->t32[cur], m->t32[1 - cur], m->P32, m->P64, a, m->tb, m->d_twork, nsteps, m->stream);
+        return launch_truth_run64(m->t64[cur], m->t64[1 - cur], m->P64, a, m->tb, m->twork.p, nsteps, m->stream);
+    return launch_truth_run32(m->t32[cur], m->t32[1 - cur], m->P32, m->P64, a, m->tb, m->twork.p, nsteps, m->stream);
 }
 
 int ms_truth_step(ms_model *m, double dt, int64_t nsteps)
