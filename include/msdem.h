@@ -256,7 +256,7 @@ int ms_time_kernel(ms_model *m, int32_t which, double dt, int32_t reps, double *
  * skin_steps fine steps (1 .. 1000); cells of at most 256 floes share a
  * block of 256 threads, a floe per thread, up to block_floes (32 .. 256)
  * floes in all (fewer where the model is too small to fill the SMs with such
- * blocks); a larger cell has a block of its own.  Floes do not depend
+ * blocks and no closure is attached); a larger cell has a block of its own.  Floes do not depend
  * on skin_steps, block_floes or the other cells of the model, and
  * neither do the moments: the per-cell sums are exact fixed-point integer
  * sums (each value relative to the largest binary exponent of its cell and
@@ -463,8 +463,11 @@ void ms_mlp_free(ms_mlp *m);
  * the measured drag, and the cell may take the closure for at most 3
  * intervals after a check whose relative error was at most tol (floor: the
  * drag of 1 cm/s on 1 m ice).  So the first interval after attaching runs
- * every cell's DEM.  Every other cell runs the particle step (the fallback).  A closure cell skips its DEM for
- * the interval: it takes its pending coarse increments at once, its velocity
+ * every cell's DEM.  With launch variant 5 the cells that share a block
+ * (ms_set_resident: up to block_floes floes of small cells in decreasing
+ * order of size, however small the model) take the closure only if every one
+ * of them that holds floes may.  Every other cell runs the particle step (the
+ * fallback).  A closure cell skips its DEM for the interval: it takes its pending coarse increments at once, its velocity
  * spread follows the predicted variance rate, and the coarse step sees the
  * predicted tendencies.  mode 2: as mode 0, but `mlp` predicts the
  * tendencies less features 12-15 (the drag at the interval's start and the

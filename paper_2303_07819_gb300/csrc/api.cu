@@ -916,9 +916,12 @@ static int build_groups(ms_model *m, CellLaunch &cl)
     // with fewer warps to wait for (16 cells of 16 floes: 1.94 us a step in
     // groups of 32, 2.34 us in one of 256; on 47,000 floes, three blocks of
     // 128 an SM, no difference).
+    // With a closure attached the groups say which cells take it together
+    // (k_group_veto), so results would depend on the number of SMs: the
+    // groups are then the caller's (ms_set_resident).
     int cap = cl.run_cap1;
     for (int c : {128, 64, 32})
-        if ((long long)m->n * 5 <= 4LL * c * m->sm_count) cap = std::min(cap, c);
+        if (!hybrid_on(m) && (long long)m->n * 5 <= 4LL * c * m->sm_count) cap = std::min(cap, c);
     std::vector<G> gs;
     const int cap_max = 4 * RUN_T;
     std::vector<std::vector<int>> by_room(cap_max + 1);   // open groups by free floes
