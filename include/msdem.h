@@ -207,9 +207,9 @@ int ms_set_stream(ms_model *m, void *stream);
 
 /* Autotune the msDEM cell kernel on the model's current state: times each
  * launch variant (pair search, threads per block, bin width) out of place
- * (the state is not changed) and keeps the fastest.  FP32 candidates are
- * timed over `reps` whole coarse intervals (ms_time_kernel which = 2), FP64
- * ones over `reps` single steps.  best_ms (host, may be NULL) receives the
+ * (the state is not changed) and keeps the fastest.  Candidates are timed
+ * over `reps` whole coarse intervals (ms_time_kernel which = 2); in FP64 with
+ * a cell above 1024 floes over `reps` single steps.  best_ms (host, may be NULL) receives the
  * fastest mean time per fine step. */
 int ms_autotune(ms_model *m, double dt, int32_t reps, double *best_ms);
 

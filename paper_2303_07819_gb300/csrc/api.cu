@@ -1946,9 +1946,10 @@ int ms_autotune(ms_model *m, double dt, int32_t reps, double *best_ms)
                     cand.push_back(c);
                 }
     }
-    // FP32: whole coarse intervals, so that variants that keep a cell
-    // resident across steps are timed by what they save
-    const int which = m->precision == MS_FP32 ? 2 : 0;
+    // Whole coarse intervals, so that kernels that keep a cell resident across
+    // steps are timed by what they save (a step alone is a launch with its
+    // loads, its search and its moments); FP64 cells that are not kept, a step.
+    const int which = m->precision == MS_FP32 || resident64(m) ? 2 : 0;
     const double per = which == 2 ? (double)m->interval : 1.0;
     const CellLaunch keep = m->cl;
     double best = 1e30;

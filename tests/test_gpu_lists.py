@@ -10,6 +10,7 @@ import time
 import numpy as np
 import pytest
 
+from paper_2303_07819_gb300.inputs import square_4x4
 from tests.conftest import ROOT
 from tests.parity import rel_errors, report
 from tests.test_gpu_runs import TOL, crowd, join, ring, soft
@@ -214,3 +215,14 @@ print("same")
 """)
     r = subprocess.run([sys.executable, str(prog)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "same" in r.stdout, r.stdout + r.stderr
+
+
+def test_fp64_autotune_times_what_a_step_makes(ms):
+    """The time ms_autotune returns and chooses by is that of the run of an
+    interval that ms_step makes, not of a step with a launch, loads, a search
+    and moments of its own."""
+    s = square_4x4()
+    m = ms.Model(s["params"], s["floes"], ms.MS_FP64)
+    best = m.autotune(s["dt"], reps=5)
+    run = min(m.time_kernel(2, s["dt"], reps=5) for _ in range(5)) / s["params"]["N0"]
+    assert 0.7 * run < best < 1.3 * run, (best, run)
