@@ -226,3 +226,33 @@ def test_fp64_autotune_times_what_a_step_makes(ms):
     best = m.autotune(s["dt"], reps=5)
     run = min(m.time_kernel(2, s["dt"], reps=5) for _ in range(5)) / s["params"]["N0"]
     assert 0.7 * run < best < 1.3 * run, (best, run)
+
+
+@pytest.mark.parametrize("nx,n,sparse", [(1, 250, False), (16, 80, False), (16, 80, True)])
+def test_fp32_blocks_of_256_that_test_every_pair(orc, ms, nx, n, sparse):
+    """Contacts alone exceed the room of a block's lists (12 candidates a floe
+    for 256 floes, 384 hits beyond a floe's first 12), with skins or without:
+    a cell of 250 floes with a block of its own, blocks of three crowded
+    cells of 80, and of crowded cells beside a sparse one."""
+    side = 25e3
+    parts, deg = [], []
+    for c in range(nx * nx):
+        f = crowd(1000 + c, n, side, 0.3 if sparse and c % 3 == 1 else 10.0)
+        dx, dy = (f[k][:, None] - f[k][None, :] for k in ("x", "y"))
+        dx, dy = dx - side * np.rint(dx / side), dy - side * np.rint(dy / side)
+        deg.append((np.hypot(dx, dy) < f["r"][:, None] + f["r"][None, :]).sum(1) - 1)
+        f["x"] += side * (c % nx)
+        f["y"] += side * (c // nx)
+        parts.append(f)
+    group = max(1, 256 // n)
+    over = []
+    for g in range(0, nx * nx - group + 1, group):
+        d = np.concatenate(deg[g:g + group])
+        over.append(d.sum() > 12 * 256 or np.maximum(d - 12, 0).sum() > 384)
+    assert np.mean(over) >= (0.5 if sparse else 1.0)
+    f, p = join(parts), dict(soft(nx, nx * side), couple=0)
+    o, m = orc.Model(p, f), ms.Model(p, f, ms.MS_FP32)
+    o.step(10.0, 12)
+    m.step(10.0, 12)
+    e = rel_errors(m.moments(), o.moments(), p, TOL[0][1])
+    assert e.max() <= TOL[0][0], report(e)
