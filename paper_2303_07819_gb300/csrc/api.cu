@@ -1128,10 +1128,12 @@ static int setup_truth_bins(ms_model *m, const double *r, double rmax)
         if (b.nscan_blocks > 1024) return fail(MS_ERR_ARG, "too many bins (%d)", nbins);
         CK(dalloc(m, &b.count, nbins));
         CK(dalloc(m, &b.start, nbins + 1));
-        CK(dalloc(m, &b.cursor, nbins));
-        CK(dalloc(m, &b.sorted, m->n));
-        CK(dalloc(m, &b.bin, m->n));
-        CK(dalloc(m, &b.scan_tmp, b.nscan_blocks));
+        if (k == 1) {
+            CK(dalloc(m, &b.cursor, nbins));
+            CK(dalloc(m, &b.sorted, m->n));
+            CK(dalloc(m, &b.bin, m->n));
+            CK(dalloc(m, &b.scan_tmp, b.nscan_blocks));
+        }
         const int nn = (int)m->n;
         CK(cudaMemcpyAsync(b.start + nbins, &nn, sizeof(int), cudaMemcpyHostToDevice, m->stream));
         CK(cudaStreamSynchronize(m->stream));

@@ -483,6 +483,7 @@ struct TruthBins {
     __host__ __device__ int nbins() const { return nbx * nby + nbx2 * nby2; }
     int *count;            // [nbins]
     int *start;            // [nbins + 1]
+    // the coarse cells' grid only (the truth steps keep theirs in their work arrays)
     int *cursor;           // [nbins]
     int *sorted;           // [n] floe indices grouped by bin
     int *bin;              // [n]
