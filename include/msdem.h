@@ -20,10 +20,9 @@
  *    ms_free: in ms_init, and by the first call of a part that not every model
  *    uses -- ms_truth_step (360 bytes a floe in FP32, 424 in FP64, and in FP64 up
  *    to 64 MB for the current), ms_time_kernel and ms_autotune (out-of-place
- *    state), ms_set_shard, ms_closure_attach.  A call whose
- *    allocation fails returns MS_ERR_CUDA and may be made again.  One model
- *    handle belongs to one host thread at a time; calls on different handles
- *    are independent.
+ *    state), ms_set_shard, ms_closure_attach.  A call whose allocation fails
+ *    returns MS_ERR_CUDA.  One model handle belongs to one host thread at a
+ *    time; calls on different handles are independent.
  *  - Every call is synchronous: when it returns, its work on the model's
  *    stream has finished and its outputs are valid.
  *  - Return value: MS_OK (0) or a negative MS_ERR_* code; ms_last_error()
@@ -189,8 +188,10 @@ int ms_coupling(ms_model *m, double *q, double *targets, double *window,
                 int64_t *flags);
 
 /* The un-localised truth DEM (Sec. 4): the same floes on the whole periodic
- * domain, advanced on the library's own copy (rebinned every step by a GPU
- * counting sort).  Same dt rule as ms_step. */
+ * domain, advanced on the library's own copy (candidate lists, made again by
+ * a GPU counting sort when a floe has moved farther than its skin; however a
+ * run of steps is split into calls, the floes are the same to the bit).  The
+ * first call allocates its work arrays.  Same dt rule as ms_step. */
 int ms_truth_step(ms_model *m, double dt, int64_t nsteps);
 
 /* Truth floes binned by the coarse cell holding their centre; same columns

@@ -17,9 +17,16 @@
 // resuming it, changes no bit.  Floes of radius <= r_split and larger ones sit
 // in separate grids of bins, as the host chose them (setup_truth_bins).
 //
-// Measured (65,341 power-law floes, FP32): 87 us a step as nine launches, 8.1 us
-// here in long runs, 78 for a call of one step with its build; 115,200 floes of
-// one size: 9.6 in long runs.
+// A skin has an upper bound (TruthBins::skin_max), so that lists stay a few
+// neighbours long at any speed, and a floe with more candidates than its list
+// holds is searched by its warp at every step (next_portion).
+//
+// Measured, us a step as nine launches and here (FP32): 65,341 power-law floes
+// in long runs 65 and 7.9, in calls of one step, with the build, 76 and 77;
+// 65,000 floes of 100-300 m with one of 9 or 19 km (125 or 265 partners), in
+// calls of 20, 93 and 23 or 189 and 41; 500 floes in a million bins, in calls
+// of one step, 61 and 52; 115,200 floes of one size in long runs 9.6.  FP64,
+// the power-law floes: 519 and 70, in calls of one step 535 and 138.
 #include <algorithm>
 #include <cfloat>
 #include <climits>
@@ -358,8 +365,8 @@ __device__ __forceinline__ void sort_warp(int *v, int m)
 // Floes with more candidates than a list holds, of one warp's 32: their
 // contacts are found by the whole warp, a candidate a lane, and handed to the
 // floe's lane in portions of up to LT, in ascending order.  (One lane
-// searching for one contact after another took 0.3 ms a step for a floe of
-// 19 km among floes of 0.2 km, the search of all bins once a step before 0.19.)
+// searching for one contact after another: 157 us a step for the floe of 19 km
+// above, 41 so.)
 struct LongLists {
     unsigned left;         // lanes whose floes are still to be searched
     int src, at, held;     // the floe's lane; the next partner to hand on, partners found
