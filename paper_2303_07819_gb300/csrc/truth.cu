@@ -86,43 +86,35 @@ __global__ void k_scatter(const int *bin, const int *start, int *cursor, int *so
     sorted[start[b] + atomicAdd(&cursor[b], 1)] = (int)l;
 }
 
-// Each bin's floe indices into ascending order, a thread per bin (grids with
-// few floes per bin): up to 16 indices sorted in registers, larger bins in
-// place in global memory.
-__global__ void k_bin_sort_sparse(const int *start, int *sorted, int nbins)
+// v[0..m) ascending, in place, by a warp: sorted runs of 1, 2, 4, ... merged in
+// pairs, the first comparison of a merge mirrored, so that every comparison
+// puts the smaller number lower and a run cut off at m needs no padding
+// (Batcher's bitonic merge in its one-directional form).
+__device__ void sort_long(int *v, int m)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nbins) return;
-    const int s = start[b], m = start[b + 1] - s;
-    if (m <= 1) return;
-    int *bin = sorted + s;
-    if (m <= 16) {
-        int v[16];
-#pragma unroll
-        for (int i = 0; i < 16; i++) v[i] = i < m ? bin[i] : INT_MAX;
-        // insertion sort on registers (the unrolled indices keep v in registers)
-#pragma unroll
-        for (int i = 1; i < 16; i++) {
-#pragma unroll
-            for (int j = i; j > 0; j--) {
-                const int lo = min(v[j - 1], v[j]), hi = max(v[j - 1], v[j]);
-                v[j - 1] = lo;
-                v[j] = hi;
+    const int lane = threadIdx.x & 31;
+    auto order = [&](long long i, long long j) {
+        if (j >= m) return;
+        const int a = v[i], b = v[j];
+        if (a > b) {
+            v[i] = b;
+            v[j] = a;
+        }
+    };
+    for (long long run = 1; run < m; run <<= 1) {
+        const long long pairs = (m + 2 * run - 1) / (2 * run) * run;
+        for (long long p = lane; p < pairs; p += 32) {
+            const long long r = p & (run - 1), first = (p - r) * 2;
+            order(first + r, first + 2 * run - 1 - r);
+        }
+        __syncwarp();
+        for (long long d = run >> 1; d > 0; d >>= 1) {
+            for (long long p = lane; p < pairs; p += 32) {
+                const long long i = 2 * p - (p & (d - 1));
+                order(i, i + d);
             }
+            __syncwarp();
         }
-#pragma unroll
-        for (int i = 0; i < 16; i++)
-            if (i < m) bin[i] = v[i];
-        return;
-    }
-    for (int i = 1; i < m; i++) {
-        const int key = bin[i];
-        int j = i - 1;
-        while (j >= 0 && bin[j] > key) {
-            bin[j + 1] = bin[j];
-            j--;
-        }
-        bin[j + 1] = key;
     }
 }
 
@@ -150,8 +142,15 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) k_bin_sort(const int *start, 
         return;
     }
     // larger bins: at most 8 entries per lane held in registers until all
-    // lanes have ranked theirs (bins above 256 floes fall back to a serial
-    // insertion sort by lane 0)
+    // lanes have ranked theirs; up to 4096 floes, the most a cell starts with, a
+    // serial insertion sort by lane 0 (the scatter leaves them nearly in order);
+    // above that, floes of a run that piled up, or a diverged FP64 state's, all
+    // of whose positions count as 0: merges by the warp, 0.1 s for 60,000 floes
+    // where insertions could take the square of that
+    if (m > 4096) {
+        sort_long(bin, m);
+        return;
+    }
     if (m > 256) {
         if (lane == 0)
             for (int i = 1; i < m; i++) {
@@ -265,10 +264,7 @@ cudaError_t counting_sort(TruthBins &b, long long n, BinF binf, cudaStream_t st)
     if ((e = bins_scan(b, nbins, st)) != cudaSuccess) return e;
     const int T = 256;
     if (n > 0) k_scatter<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.bin, b.start, b.cursor, b.sorted, n);
-    if (n < 4LL * nbins)   // few floes per bin on average: a thread per bin
-        k_bin_sort_sparse<<<(nbins + T - 1) / T, T, 0, st>>>(b.start, b.sorted, nbins);
-    else
-        k_bin_sort<<<(nbins + SORT_WARPS - 1) / SORT_WARPS, SORT_WARPS * 32, 0, st>>>(b.start, b.sorted, nbins);
+    k_bin_sort<<<(nbins + SORT_WARPS - 1) / SORT_WARPS, SORT_WARPS * 32, 0, st>>>(b.start, b.sorted, nbins);
     return cudaGetLastError();
 }
 

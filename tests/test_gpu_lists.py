@@ -256,3 +256,53 @@ def test_fp32_blocks_of_256_that_test_every_pair(orc, ms, nx, n, sparse):
     m.step(10.0, 12)
     e = rel_errors(m.moments(), o.moments(), p, TOL[0][1])
     assert e.max() <= TOL[0][0], report(e)
+
+
+@pytest.mark.parametrize("n", [4096, 4097, 8192, 100_003, 200_000])
+def test_moments_of_a_crowded_cell(ms, n):
+    """Nearly all floes in one cell, around the 4096 above which a warp merges
+    its list, through the allocation-free entry point: the sums of each
+    cell's floes, the same twice."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n)
+    side, extra = 25e3, 37
+    p = dict(soft(2, 2 * side))
+    f = {k: rng.uniform(0.5, 1.5, n + extra) for k in ("u", "v", "omega", "r", "h")}
+    f["x"] = np.r_[rng.uniform(0, side, n), rng.uniform(side, 2 * side, extra)]
+    f["y"] = rng.uniform(0, side, n + extra)
+    order = rng.permutation(n + extra)
+    dev = {k: torch.tensor(v[order], dtype=torch.float64, device="cuda") for k, v in f.items()}
+    fd = torch.tensor(rng.normal(size=(3, n + extra)), dtype=torch.float64, device="cuda")
+    out = []
+    for _ in range(2):
+        o = torch.full((4, 12), float("nan"), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        ms.cell_moments_noalloc(p, n + extra, *(dev[k].data_ptr() for k in ("x", "y", "u", "v", "omega", "r", "h")),
+                                fd.data_ptr(), o.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        assert time.perf_counter() - t < 1.0
+        out.append(o.cpu().numpy())
+    assert np.array_equal(out[0], out[1])
+    m = p["rho_ice"] * np.pi * f["r"] ** 2 * f["h"]
+    d = fd.cpu().numpy()[:, np.argsort(order)]
+    for c, sel in ((0, slice(0, n)), (1, slice(n, n + extra))):
+        ref = [m[sel].sum(), (m * f["u"])[sel].sum(), (m * f["v"])[sel].sum()]
+        assert out[0][c, 0] == (n if c == 0 else extra)
+        assert np.allclose(out[0][c, 1:4], ref, rtol=1e-11, atol=0)
+        assert np.allclose(out[0][c, 9:12], d[:, sel].sum(1), rtol=1e-10, atol=1e-10)
+    assert np.all(out[0][2:] == 0)
+
+
+def test_moments_of_a_diverged_truth_state(ms):
+    """The moments of a truth DEM whose FP64 positions are NaN, so that all
+    floes count to one cell: an answer in a time of the order of a step's."""
+    n, L = 60_000, 300e3
+    f, p = packed(n, L), dict(soft(8, L), couple=0)
+    f["u"][:] = 1.0e12
+    m = ms.Model(p, f, ms.MS_FP64)
+    with pytest.raises(ms.MsError):
+        m.truth_step(10.0, 100)
+    t = time.perf_counter()
+    mom = m.truth_moments()
+    assert time.perf_counter() - t < 1.0
+    assert mom[:, 0].sum() == n
