@@ -167,21 +167,28 @@ __device__ __forceinline__ bool contact_add(R dx, R dy, R d2, R rl, R rj, R hl, 
 // Ocean drag at the floe plus wind drag, Eq. (2.1c-d): translation
 // alpha (u - v)|u - v| with alpha = Cd rho_o pi r^2 (wind: Ca rho_a pi r^2),
 // rotation beta (zeta/2 - w)|zeta/2 - w| with beta = Cd rho_o pi r^4.
-template <class R>
+// norm(a, b): the length of (a, b).
+template <class R, class Norm>
 __device__ __forceinline__ void drag_force(const Phys<R> &P, R uo, R vo, R zeta, R ua, R va,
-                                           R u, R v, R w, R r, R &Fx, R &Fy, R &T)
+                                           R u, R v, R w, R r, R &Fx, R &Fy, R &T, Norm &&norm)
 {
     const R ao = P.drag_o * r * r;
     const R aa = P.drag_a * r * r;
     const R bo = P.drag_o * r * r * r * r;
     const R du = uo - u, dv = vo - v;
-    const R so = sqrt(du * du + dv * dv);
+    const R so = norm(du, dv);
     const R au = ua - u, av = va - v;
-    const R sa = sqrt(au * au + av * av);
+    const R sa = norm(au, av);
     const R dw = R(0.5) * zeta - w;
     Fx = ao * du * so + aa * au * sa;
     Fy = ao * dv * so + aa * av * sa;
     T = bo * dw * fabs(dw);
+}
+template <class R>
+__device__ __forceinline__ void drag_force(const Phys<R> &P, R uo, R vo, R zeta, R ua, R va,
+                                           R u, R v, R w, R r, R &Fx, R &Fy, R &T)
+{
+    drag_force(P, uo, vo, zeta, ua, va, u, v, w, r, Fx, Fy, T, [](R a, R b) { return sqrt(a * a + b * b); });
 }
 
 // Ocean current and its curl at a global position, FP64 (mode coefficients

@@ -242,6 +242,12 @@ __device__ __forceinline__ void ocean_at(const Phys<double> &P, const Work<Tr64>
     }
 }
 
+// |(x, y)| of the drag.  In FP64 the rounding is written out: which of the two
+// squares the compiler fuses depends on the code around it, and the last bits
+// of every floe with it.
+__device__ __forceinline__ float length(float x, float y) { return sqrtf(x * x + y * y); }
+__device__ __forceinline__ double length(double x, double y) { return sqrt(__fma_rn(x, x, __dmul_rn(y, y))); }
+
 __global__ void k_truth_tiles(Phys<double> P, Geom g, Work<Tr64> w)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -675,7 +681,8 @@ k_truth_run(typename T::State in, typename T::State out, Phys<typename T::R> P, 
             ocean_at(P, w, a, me, uo, vo, zeta);
             if (walls) wall_force(me, a, q.u, q.v, q.w, P, fx, fy, tq, deep);
             R Fdx, Fdy, Td;
-            drag_force(P, uo, vo, zeta, (R)wa.x, (R)wa.y, q.u, q.v, q.w, me.r, Fdx, Fdy, Td);
+            drag_force(P, uo, vo, zeta, (R)wa.x, (R)wa.y, q.u, q.v, q.w, me.r, Fdx, Fdy, Td,
+                       [](R x, R y) { return length(x, y); });
             fx += Fdx; fy += Fdy; tq += Td;
             const R dt = (R)a.dt;
             const R m = P.mass_c * me.r * me.r * me.h;
